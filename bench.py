@@ -207,11 +207,9 @@ def barrier(world):
         dist.barrier()
 
 
+FINE_SOURCES = ["paper_2404_02521_gb300/csrc/" + f for f in ("fine.cu", "fine_tile.cuh", "fine_launch.cuh", "common.cuh")]
 KERNEL_SOURCES = {
-    "fine_ctile_kernel": ["paper_2404_02521_gb300/csrc/fine.cu", "paper_2404_02521_gb300/csrc/band.cuh",
-                          "paper_2404_02521_gb300/csrc/common.cuh"],
-    "fine_band_kernel": ["paper_2404_02521_gb300/csrc/fine.cu", "paper_2404_02521_gb300/csrc/band.cuh",
-                         "paper_2404_02521_gb300/csrc/common.cuh"],
+    "fine_tile_kernel": FINE_SOURCES,
     "sweep_band_kernel": ["paper_2404_02521_gb300/csrc/coarse.cu", "paper_2404_02521_gb300/csrc/band.cuh",
                           "paper_2404_02521_gb300/csrc/common.cuh"],
 }
@@ -344,15 +342,15 @@ def large_arm(args, world, local):
     chunks = sum((N - kk + 95) // 96 for k in ks for kk in range(k))
     avg_states = slices_f / max(1, chunks)
     # DRAM bytes per launch: the committed capture's bytes per state and launch x avg_states
-    ent = traffic_entry("fine_ctile_kernel")
+    ent = traffic_entry("fine_tile_kernel")
     traffic = ent["dram_bytes_per_state_launch"] * avg_states if ent else None
     hbm_peak = float(pk.get("hbm_gbs", 6800.0))
     alg_bytes_launch = avg_states * M * M * FINE_ALG_BYTES_PER_POINT_LAUNCH
-    roof = {"kernel": "fine_ctile_kernel", "bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+    roof = {"kernel": "fine_tile_kernel", "bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak, "traffic": traffic,
             "peak_source": f"FP32 lanes x 2 x {sm_max:.0f} MHz of {sms} SMs ({pk_kind} max clock)"}
     kernels = {
-        "fine_ctile_kernel": {
+        "fine_tile_kernel": {
             "ms_total": phases["fine_ms"], "launches": phases["fine_launches"], "ms_per_launch": ms_per_launch,
             "states_per_launch": avg_states, "bound": "alu", "achieved_tflops": achieved, "peak_tflops": peak,
             "frac": achieved / peak,
@@ -577,7 +575,7 @@ def exchange_arm(args, local):
             "krylov_iters_per_solve": krylov_iters / len(problems),
             "us_per_krylov_iter": 1e3 * phases["coarse_ms"] / max(1, args.steps * krylov_iters),
             "note": "serial coarse sweep on one thread-block cluster: latency-bound"},
-        "fine_band_kernel": {"ms_total": phases["fine_ms"], "launches": phases["fine_launches"]},
+        "fine_tile_kernel": {"ms_total": phases["fine_ms"], "launches": phases["fine_launches"]},
     }
 
 

@@ -108,7 +108,8 @@ int bs_payoff(const bs_grid* g, const bs_params* p, float* u, bs_stream stream);
  * enqueues kernels, so after one call with the same grid and batch it can be captured into
  * a CUDA graph.
  * Errors: BS_ERR_ARG (NULL, B < 1, dtau <= 0), BS_ERR_CUDA.  A BiCGSTAB step that hits its
- * iteration cap is reported by the next synchronous call on this grid as BS_ERR_NOCONV. */
+ * iteration cap is reported by the next synchronous call on this grid as BS_ERR_NOCONV, and a
+ * timed-out exchange between a cluster's CTAs (waits are bounded) as BS_ERR_CUDA. */
 int fine_propagate_batched(const bs_grid* g, const bs_params* p,
                            const float* const* u_in, float* const* u_out,
                            const double* tau0, const double* dtau, int nsteps, int B,
@@ -314,14 +315,12 @@ int bs_fine_sweeps(const bs_grid* g, const bs_params* p, double dtau, int first_
  *                        and, where their shared memory allows, use a polynomial
  *                        preconditioner and quadratic initial-guess extrapolation (all solve
  *                        the same systems to the same Krylov tolerance).
- *  BS_OPT_FINE_TILE      layout of the fine stepper: 0 (default) per launch, the one with less
- *                        work counted in waves of co-resident clusters; 1 or 2 forces one.
- *                        Grids with M > 256 run as overlapping cluster tiles: layout 1 on
- *                        regions of 256 x 256 nodes (8 CTAs, up to 24 sweeps per launch),
- *                        layout 2 on regions of 288 x 288 (9 CTAs, up to 16 sweeps).  Grids
- *                        with 128 < M <= 256 keep a state in one cluster: layout 1 on 8 CTAs
- *                        of 32 rows, layout 2 on 16 CTAs of 16 rows (one CTA per SM; faster
- *                        for one or a few states).  Smaller grids have one layout.  All
+ *  BS_OPT_FINE_TILE      layout of the fine stepper: 0 (default) per launch, the one with the least
+ *                        estimated time in waves of co-resident clusters; 1 or 2 forces one.
+ *                        Grids with M <= 256 keep a state in one cluster for all steps: layout 1
+ *                        on CTAs of 32 rows, layout 2 on CTAs of 16 rows (faster for one or a
+ *                        few states).  Grids with M > 256 run as overlapping regions: layout 1
+ *                        of 256 x 256 nodes (8 CTAs), layout 2 of 256 x 288 (9 CTAs).  All
  *                        layouts give the same result bit for bit.
  * Returns BS_OK or BS_ERR_ARG for an unknown option or an out-of-range value. */
 enum { BS_OPT_FINE_SWEEPS = 0, BS_OPT_JACOBI_TARGET = 1, BS_OPT_KRYLOV_TOL = 2,

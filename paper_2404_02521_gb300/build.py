@@ -24,7 +24,8 @@ FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", 
 # the fine stepper's device code, too: its layouts and launch plans instantiate the same
 # stencil in different kernels, and only without implicit contraction do they round alike
 # (its multiply-adds are written as explicit fused operations)
-FILE_FLAGS = {"fine.cu": ["-fmad=false"]}
+FILE_FLAGS = {f: ["-fmad=false"] for f in ("fine.cu", "fine_wa.cu", "fine_wb.cu", "fine_wc.cu", "fine_wd.cu",
+                                           "fine_we.cu")}
 
 
 def nvcc() -> str:

@@ -752,7 +752,7 @@ int parareal_solve(const bs_grid* gc, const bs_params* p, int N, int fine_steps,
       g->ms_fine += ms_f;
       g->ms_coarse += ms_c;
       if (hstat & 2)
-        return set_error(BS_ERR_CUDA, "parareal_solve: a cluster exchange of the coarse sweep timed out");
+        return set_error(BS_ERR_CUDA, "parareal_solve: a cluster exchange timed out");
       return set_error(BS_ERR_NOCONV, "parareal_solve: a coarse BiCGSTAB solve hit its iteration cap");
     }
     if (host[0] <= tol) {

@@ -28,6 +28,7 @@
 #include <utility>
 
 #include "band.cuh"
+#include "cluster_async.cuh"
 
 namespace bsp {
 
@@ -207,52 +208,6 @@ struct KrylovFin {
 // the round r halo rows; halo rows of v are double-buffered by iteration parity since they
 // are read once more after the following round).
 // ---------------------------------------------------------------------------------------
-constexpr int kXchgWaitPolls = 1 << 22;   // bound on mbarrier polls per round
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ uint32_t cluster_addr(uint32_t local, int rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(local), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void mbar_init(uint64_t* mb, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(mb)), "r"(count) : "memory");
-}
-// the local arrival of a round, announcing the bytes the round's stores will complete
-__device__ __forceinline__ void mbar_arm(uint64_t* mb, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_addr(mb)), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_test(uint64_t* mb, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_addr(mb)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ void st_async_f32(uint32_t dst, float v, uint32_t mb) {
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];\n" ::"r"(dst),
-               "r"(__float_as_uint(v)), "r"(mb)
-               : "memory");
-}
-__device__ __forceinline__ void st_async_v2(uint32_t dst, float a, float b, uint32_t mb) {
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];\n" ::"r"(dst),
-               "r"(__float_as_uint(a)), "r"(__float_as_uint(b)), "r"(mb)
-               : "memory");
-}
-__device__ __forceinline__ void st_async_v4(uint32_t dst, float a, float b, float c, float d, uint32_t mb) {
-  asm volatile(
-      "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];\n" ::"r"(dst),
-      "r"(__float_as_uint(a)), "r"(__float_as_uint(b)), "r"(__float_as_uint(c)), "r"(__float_as_uint(d)),
-      "r"(mb)
-      : "memory");
-}
-
 struct Xchg {
   uint64_t* mb;     // [2] mbarriers (one per round parity), arrival count 1
   float* kslot;     // [2][kMaxCluster][4] partial sums by source rank

@@ -166,7 +166,7 @@ __device__ __forceinline__ void row_coefs(const ItemDesc& d, int j, float& cs, f
 __device__ __forceinline__ float inv_diag(const ItemDesc& d, int i, int j) {
   const float fi = (float)i, fj = (float)j;
   const float diag = 1.0f + (2.0f * (d.ax * (fi * fi)) + 2.0f * (d.ay * (fj * fj)) + d.rdt);
-  return 1.0f / diag;
+  return __frcp_rn(diag);   // the correctly rounded quotient 1 / diag, without the division's slow path
 }
 
 // ---------------------------------------------------------------------------------------
@@ -308,7 +308,8 @@ int resampled_launches_per_slice();
 // Pipelined driver: whether N slices are enough to pipeline, and the slices per chunk.
 bool pipeline_eligible(int N);
 int pipeline_chunk(bs_grid* g, const ItemDesc& dc, int N, cudaStream_t s, int* S);
-int fine_cluster_capacity(const bs_grid* g);   // fine band clusters the device runs at once (0: unknown)
+int fine_cluster_capacity(const bs_grid* g);   // fine clusters (M <= 256) the device runs at once (0: unknown)
+int fine_cluster_ctas(const bs_grid* g);       // CTAs of such a cluster
 int coarse_cluster_ctas(const bs_grid* g, const ItemDesc& d, cudaStream_t s, int* ctas);
 int coarse_variant_info(int v, int M, int* ctas, int* threads, int* rows, int* poly, int* quad);
 int parareal_pipelined(bs_grid* g, const bs_params* p, int N, int fine_steps, int coarse_steps, double tol,

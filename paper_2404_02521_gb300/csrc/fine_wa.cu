@@ -1,0 +1,7 @@
+// Instances of the fine tile kernel (columns and rows per lane); see fine_tile.cuh.
+#include "fine_launch.cuh"
+
+namespace bsp {
+BS_FINE_INSTANCE(2, 4)
+BS_FINE_INSTANCE(4, 4)
+}  // namespace bsp

@@ -104,7 +104,7 @@ int pipeline_chunk(bs_grid* g, const ItemDesc& dc, int N, cudaStream_t s, int* S
     int cc = 0;
     int rc = coarse_cluster_ctas(g, dc, s, &cc);
     if (rc) return rc;
-    const int cf = g->shape.C;
+    const int cf = fine_cluster_ctas(g);
     const int wave = cap - (cc + cf - 1) / cf;
     if (wave >= 1 && wave < quarter) quarter = wave;
   }
@@ -278,7 +278,7 @@ int parareal_pipelined(bs_grid* g, const bs_params* p, int N, int fine_steps, in
       *k_done = k + 1;
       BS_CUDA_TRY(cudaStreamSynchronize(sf));
       if (hstat & 2)
-        return set_error(BS_ERR_CUDA, "parareal_solve: a cluster exchange of the coarse sweep timed out");
+        return set_error(BS_ERR_CUDA, "parareal_solve: a cluster exchange timed out");
       return set_error(BS_ERR_NOCONV, "parareal_solve: a coarse BiCGSTAB solve hit its iteration cap");
     }
     if (host <= tol) {
