@@ -32,49 +32,25 @@
 
 namespace bsp {
 
-// The pointwise phases of a step (one launch each): INIT copies u_in into (hi, lo = 0) and
-// zeroes the increment; FACE writes the far-face data at tau; RHS forms b = dtau R_h hi;
-// APPLY adds the increment to (hi, lo); OUT writes hi + lo.
-__global__ void __launch_bounds__(kF3Threads) f3_phase_kernel(const __grid_constant__ F3Batch fb, int phase,
-                                                              int step, int cur) {
+// The pointwise passes of a propagation: INIT copies u_in into (hi, lo = 0), zeroes the increment
+// and sets the far faces of the first step; OUT writes hi + lo.
+enum { F3_INIT = 0, F3_OUT = 1 };
+__global__ void __launch_bounds__(kF3Threads) f3_phase_kernel(const __grid_constant__ F3Batch fb, int phase, int nsteps) {
   const F3Item& it = fb.it[blockIdx.y];
   const int M = fb.M, n3 = M * M * M;
   const int e = blockIdx.x * kF3Threads + threadIdx.x;
   if (e >= n3) return;
+  if (phase == F3_OUT) {
+    it.out[e] = it.hi[e] + it.lo[e];
+    return;
+  }
   int i, j, k;
   f3_node(e, M, i, j, k);
   const bool pde = i < M - 1 && j < M - 1 && k < M - 1;
-  float* d = cur ? it.dB : it.dA;
-  switch (phase) {
-    case F3_INIT:
-      it.hi[e] = it.in[e];
-      it.lo[e] = 0.f;
-      it.dA[e] = 0.f;
-      it.dB[e] = 0.f;
-      break;
-    case F3_FACE:
-      if (!pde) {
-        it.hi[e] = f3_far_field(fb, i, j, k, it.tau0 + (step + 1) * fb.dtau);
-      }
-      break;
-    case F3_RHS:
-      it.b[e] = pde ? f3_offdiag(it.hi, fb.c, M, i, j, k) - (f3_diag(fb.c, i, j, k) - 1.0f) * it.hi[e] : 0.f;
-      break;
-    case F3_APPLY:
-      if (pde) {
-        const float h0 = it.hi[e], v = d[e];
-        const float s = h0 + v, bb = s - h0;
-        const float err = (h0 - (s - bb)) + (v - bb);
-        const float l = it.lo[e] + err;
-        const float hn = s + l;
-        it.lo[e] = l - (hn - s);
-        it.hi[e] = hn;
-      }
-      break;
-    case F3_OUT:
-      it.out[e] = it.hi[e] + it.lo[e];
-      break;
-  }
+  it.hi[e] = pde || nsteps == 0 ? it.in[e] : f3_far_field(fb, i, j, k, it.tau0 + fb.dtau);
+  it.lo[e] = 0.f;
+  it.dA[e] = 0.f;
+  it.dB[e] = 0.f;
 }
 
 // Asynchronous 4-byte global -> shared copy (all of a thread's copies in flight at once);
@@ -88,26 +64,6 @@ __device__ __forceinline__ void f3_cp_async4(float* dst, const float* src, bool 
 // node on every side, i fastest.  Entries outside the grid are 0 (their weights are 0 too).
 constexpr int kHI = kF3TileI + 2, kHJ = kF3TileJ + 2, kHK = kF3PlanesPerBlock + 2;
 constexpr int kTileFloats = kHI * kHJ * kHK;
-
-// Off-diagonal part of dtau R_h at the node of tile index L (column coefficients precomputed;
-// no guards: a neighbour at index -1 is 0 in the tile and has weight 0).
-struct F3Col {
-  float wxp, wxm, wyp, wym, cxy, cxz, cyz;
-};
-__device__ __forceinline__ float f3_tile_offdiag(const float* t, int L, const F3Col& w, float az, float mz,
-                                                 float fk) {
-  constexpr int X = 1, Y = kHI, Z = kHI * kHJ;
-  float acc = w.wxp * t[L + X];
-  acc = fmaf(w.wxm, t[L - X], acc);
-  acc = fmaf(w.wyp, t[L + Y], acc);
-  acc = fmaf(w.wym, t[L - Y], acc);
-  acc = fmaf(az + mz, t[L + Z], acc);
-  acc = fmaf(az - mz, t[L - Z], acc);
-  acc = fmaf(w.cxy, (t[L + X + Y] + t[L - X - Y]) - (t[L + X - Y] + t[L - X + Y]), acc);
-  acc = fmaf(w.cxz * fk, (t[L + X + Z] + t[L - X - Z]) - (t[L + X - Z] + t[L - X + Z]), acc);
-  acc = fmaf(w.cyz * fk, (t[L + Y + Z] + t[L - Y - Z]) - (t[L + Y - Z] + t[L - Y + Z]), acc);
-  return acc;
-}
 
 // One Jacobi sweep: d_new = (b + offdiag(d_old)) / diag at PDE nodes, 0 elsewhere.  A block
 // stages its halo tile of d_old in shared memory (asynchronous copies, coalesced along i),
@@ -191,12 +147,12 @@ __global__ void __launch_bounds__(kF3TileI * kF3TileJ, 4) f3_sweep_kernel(const 
     const float diag = dxy + 2.0f * az;
     float bv;
     if (first) {   // RHS: b = offdiag(hi) - (diag - 1) hi
-      bv = f3_tile_offdiag(sh, L, w, az, mz, fk) - (diag - 1.0f) * sh[L];
+      bv = f3_tile_offdiag<kHI, kHJ>(sh, L, w, az, mz, fk) - (diag - 1.0f) * sh[L];
       it.b[e] = bv;
     } else {
       bv = bq[kk];
     }
-    const float dn = (bv + f3_tile_offdiag(sd, L, w, az, mz, fk)) / diag;
+    const float dn = (bv + f3_tile_offdiag<kHI, kHJ>(sd, L, w, az, mz, fk)) / diag;
     dout[e] = dn;
     if (last) {   // APPLY: compensated add of the increment
       const float h0 = hq[kk];
@@ -257,11 +213,10 @@ double f3_contraction(int M, const bs_params3& p, double dtau) {
   return q;
 }
 
-static int f3_sweeps(double q, bool cold) {
-  const double target = cold ? 1.0 / 4194304.0 : 1.0 / 1024.0;
+static int f3_sweeps(double q, int step) {
+  const double target = step == 0 ? 1.0 / 4194304.0 : 1.0 / 1024.0;
   if (q <= 0.0) return 2;
-  const int m = (int)std::ceil(std::log(target) / std::log(q));
-  return m < 2 ? 2 : m;
+  return std::max(2, (int)std::ceil(std::log(target) / std::log(q)));
 }
 
 int f3_check(int M, double xmax, const bs_params3* p) {
@@ -349,7 +304,6 @@ int fine_propagate3(int M, double xmax, const bs_params3* p, const float* const*
   const double q = f3_contraction(M, *p, dtau);
   if (!(q < 0.8))
     return set_error(BS_ERR_ARG, "fine_propagate3: Jacobi bound %.3f >= 0.8 (take smaller steps)", q);
-  const int m0 = f3_sweeps(q, true), m1 = f3_sweeps(q, false);
   cudaStream_t s = (cudaStream_t)stream;
   const size_t n3 = (size_t)M * M * M;
   const unsigned blocks = (unsigned)((n3 + kF3Threads - 1) / kF3Threads);
@@ -377,11 +331,10 @@ int fine_propagate3(int M, double xmax, const bs_params3* p, const float* const*
     const dim3 sgrid((unsigned)(tiles_i * tiles_j), (unsigned)((M + kF3PlanesPerBlock - 1) / kF3PlanesPerBlock),
                      (unsigned)nb);
     const dim3 sblock(kF3TileI, kF3TileJ);
-    f3_phase_kernel<<<grid, kF3Threads, 0, s>>>(fb, F3_INIT, 0, 0);
-    if (nsteps > 0) f3_phase_kernel<<<grid, kF3Threads, 0, s>>>(fb, F3_FACE, 0, 0);
+    f3_phase_kernel<<<grid, kF3Threads, 0, s>>>(fb, F3_INIT, nsteps);
     int cur = 0;   // 0: the increment is in dA
     for (int step = 0; step < nsteps; ++step) {
-      const int m = step == 0 ? m0 : m1;   // >= 2
+      const int m = f3_sweeps(q, step);   // >= 2
       for (int sw = 0; sw < m; ++sw) {
         const int face_step = step + 1 < nsteps ? step + 1 : -1;
         if (sw == 0)
@@ -393,7 +346,7 @@ int fine_propagate3(int M, double xmax, const bs_params3* p, const float* const*
         cur ^= 1;
       }
     }
-    f3_phase_kernel<<<grid, kF3Threads, 0, s>>>(fb, F3_OUT, nsteps, cur);
+    f3_phase_kernel<<<grid, kF3Threads, 0, s>>>(fb, F3_OUT, nsteps);
     BS_CUDA_TRY(cudaGetLastError());
     BS_CUDA_TRY(cudaFreeAsync(ws, s));
   }

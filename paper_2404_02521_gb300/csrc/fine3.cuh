@@ -58,57 +58,36 @@ __device__ __forceinline__ float f3_far_field(const F3Batch& fb, int i, int j, i
   return far_field(fb.ex, x, y, tau);
 }
 
-// Off-diagonal part of dtau R_h applied to y at a PDE node (i, j, k <= M-2): the 18
-// neighbours; a neighbour at index -1 has weight 0 and is not read.
-__device__ __forceinline__ float f3_offdiag(const float* __restrict__ y, const F3Coef& c, int M, int i, int j,
-                                            int k) {
-  const int e = (k * M + j) * M + i;
-  const int sx = 1, sy = M, sz = M * M;
-  const float fi = (float)i, fj = (float)j, fk = (float)k;
-  const float ax = c.A[0] * (fi * fi), ay = c.A[1] * (fj * fj), az = c.A[2] * (fk * fk);
-  const float mx = c.D[0] * fi, my = c.D[1] * fj, mz = c.D[2] * fk;
-  float acc = (ax + mx) * __ldg(y + e + sx) + (ay + my) * __ldg(y + e + sy) + (az + mz) * __ldg(y + e + sz);
-  if (i > 0) acc = fmaf(ax - mx, __ldg(y + e - sx), acc);
-  if (j > 0) acc = fmaf(ay - my, __ldg(y + e - sy), acc);
-  if (k > 0) acc = fmaf(az - mz, __ldg(y + e - sz), acc);
-  // cross pairs: +(++ and --) - (+- and -+)
-  {
-    float s = __ldg(y + e + sx + sy);
-    if (i > 0 && j > 0) s += __ldg(y + e - sx - sy);
-    if (j > 0) s -= __ldg(y + e + sx - sy);
-    if (i > 0) s -= __ldg(y + e - sx + sy);
-    acc = fmaf(c.Cxy * (fi * fj), s, acc);
-  }
-  {
-    float s = __ldg(y + e + sx + sz);
-    if (i > 0 && k > 0) s += __ldg(y + e - sx - sz);
-    if (k > 0) s -= __ldg(y + e + sx - sz);
-    if (i > 0) s -= __ldg(y + e - sx + sz);
-    acc = fmaf(c.Cxz * (fi * fk), s, acc);
-  }
-  {
-    float s = __ldg(y + e + sy + sz);
-    if (j > 0 && k > 0) s += __ldg(y + e - sy - sz);
-    if (k > 0) s -= __ldg(y + e + sy - sz);
-    if (j > 0) s -= __ldg(y + e - sy + sz);
-    acc = fmaf(c.Cyz * (fj * fk), s, acc);
-  }
+// Off-diagonal part of dtau R_h at the node of index L of a shared-memory tile with HI entries
+// along i and HJ along j (column coefficients precomputed; no guards: a neighbour at index -1 is
+// 0 in the tile and has weight 0).
+struct F3Col {
+  float wxp, wxm, wyp, wym, cxy, cxz, cyz;
+};
+template <int HI, int HJ>
+__device__ __forceinline__ float f3_tile_offdiag(const float* t, int L, const F3Col& w, float az, float mz, float fk) {
+  constexpr int X = 1, Y = HI, Z = HI * HJ;
+  float acc = w.wxp * t[L + X];
+  acc = fmaf(w.wxm, t[L - X], acc);
+  acc = fmaf(w.wyp, t[L + Y], acc);
+  acc = fmaf(w.wym, t[L - Y], acc);
+  acc = fmaf(az + mz, t[L + Z], acc);
+  acc = fmaf(az - mz, t[L - Z], acc);
+  acc = fmaf(w.cxy, (t[L + X + Y] + t[L - X - Y]) - (t[L + X - Y] + t[L - X + Y]), acc);
+  acc = fmaf(w.cxz * fk, (t[L + X + Z] + t[L - X - Z]) - (t[L + X - Z] + t[L - X + Z]), acc);
+  acc = fmaf(w.cyz * fk, (t[L + Y + Z] + t[L - Y - Z]) - (t[L + Y - Z] + t[L - Y + Z]), acc);
   return acc;
-}
-
-__device__ __forceinline__ float f3_diag(const F3Coef& c, int i, int j, int k) {
-  const float fi = (float)i, fj = (float)j, fk = (float)k;
-  return 1.0f + 2.0f * (c.A[0] * (fi * fi) + c.A[1] * (fj * fj) + c.A[2] * (fk * fk)) + c.rdt;
 }
 
 // host helpers (fine3.cu)
 int f3_check(int M, double xmax, const bs_params3* p);                 // BS_OK or BS_ERR_ARG
 F3Batch f3_batch(int M, double xmax, const bs_params3& p, double dtau);  // coefficients of one step
 double f3_contraction(int M, const bs_params3& p, double dtau);         // Gershgorin bound q
-enum { F3_INIT = 0, F3_FACE = 1, F3_RHS = 2, F3_APPLY = 3, F3_OUT = 4 };
-__global__ void f3_phase_kernel(const __grid_constant__ F3Batch fb, int phase, int step, int cur);
 // G over one slice for one state, BiCGSTAB per implicit step (krylov3.cu)
+size_t k3_workspace_bytes(int M);
+int* k3_status(void* ws, int M);                                     // device int, zeroed by the caller
 int coarse_propagate3_krylov(int M, double xmax, const bs_params3& p, const float* u_in, float* u_out, double tau0,
-                             double dtau, int nsteps, double tol, int maxit, cudaStream_t s);
+                             double dtau, int nsteps, double tol, int maxit, void* ws, cudaStream_t s);
+int k3_result(void* ws, int M, int maxit, cudaStream_t s);           // synchronous
 
 }  // namespace bsp

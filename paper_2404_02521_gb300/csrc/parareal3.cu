@@ -54,13 +54,23 @@ __global__ void __launch_bounds__(kP3Threads) p3_correct_kernel(int mode, size_t
   }
 }
 
-// norms[2 n] = ||u_n||^2, norms[2 n + 1] = ||du_n||^2 from the block partials (fixed order).
+// norms[2 n] = ||u_n||^2, norms[2 n + 1] = ||du_n||^2 from the block partials (fixed order: lane by
+// lane, then a butterfly).
 __global__ void p3_sum_kernel(const double* partials, int nblocks, double* norms) {
-  if (threadIdx.x != 0) return;
   double a = 0.0, b = 0.0;
-  for (int i = 0; i < nblocks; ++i) { a += partials[2 * i]; b += partials[2 * i + 1]; }
-  norms[0] = a;
-  norms[1] = b;
+  for (int i = threadIdx.x; i < nblocks; i += 32) {
+    a += partials[2 * i];
+    b += partials[2 * i + 1];
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, off);
+    b += __shfl_xor_sync(0xffffffffu, b, off);
+  }
+  if (threadIdx.x == 0) {
+    norms[0] = a;
+    norms[1] = b;
+  }
 }
 
 }  // namespace bsp
@@ -85,8 +95,9 @@ extern "C" int parareal_solve3(int M, double xmax, const bs_params3* p, double T
   const size_t fbytes = ((2 * (size_t)N + 1) * n3 * sizeof(float) + 255) / 256 * 256;
   unsigned char* ws = nullptr;
   note_device_alloc();
-  BS_CUDA_TRY(cudaMallocAsync((void**)&ws, fbytes + (size_t)nblocks * 2 * sizeof(double) +
-                                               (size_t)(N + 1) * 2 * sizeof(double), s));
+  const size_t dbytes = ((size_t)nblocks * 2 + (size_t)(N + 1) * 2) * sizeof(double);
+  const size_t goff = (fbytes + dbytes + 255) / 256 * 256;   // the coarse solver's workspace
+  BS_CUDA_TRY(cudaMallocAsync((void**)&ws, goff + k3_workspace_bytes(M), s));
   float* Fb = reinterpret_cast<float*>(ws);
   float* Gold = Fb + (size_t)N * n3;
   float* Gnew = Gold + (size_t)N * n3;
@@ -96,7 +107,7 @@ extern "C" int parareal_solve3(int M, double xmax, const bs_params3* p, double T
   auto U = [&](int n) { return u_out + (size_t)n * n3; };
   auto G = [&](int n, float* out) -> int {   // G(u_n) over slice n: BiCGSTAB per coarse step
     return coarse_propagate3_krylov(M, xmax, *p, U(n), out, n * slice, dtg, coarse_steps, g_opt.krylov_tol,
-                                    g_opt.krylov_maxit, s);
+                                    g_opt.krylov_maxit, ws + goff, s);
   };
   auto correct = [&](int mode, int n) -> int {
     p3_correct_kernel<<<nblocks, kP3Threads, 0, s>>>(mode, n3, U(n + 1), Fb + (size_t)n * n3, Gnew,
@@ -109,10 +120,13 @@ extern "C" int parareal_solve3(int M, double xmax, const bs_params3* p, double T
     cudaFreeAsync(ws, s);
     return code;
   };
+  if (cudaMemsetAsync(k3_status(ws + goff, M), 0, sizeof(int), s) != cudaSuccess)
+    return fail(cuda_error(cudaGetLastError(), "parareal_solve3"));
   // initial sweep: u_{n+1} = G(u_n)
   for (int n = 0; n < N; ++n) {
     if ((rc = G(n, Gnew)) || (rc = correct(0, n))) return fail(rc);
   }
+  if ((rc = k3_result(ws + goff, M, g_opt.krylov_maxit, s))) return fail(rc);
   int k = 0;
   bool converged = false;
   std::vector<const float*> fin((size_t)N);
@@ -142,6 +156,7 @@ extern "C" int parareal_solve3(int M, double xmax, const bs_params3* p, double T
             cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
       return fail(cuda_error(cudaGetLastError(), "parareal_solve3"));
+    if ((rc = k3_result(ws + goff, M, g_opt.krylov_maxit, s))) return fail(rc);
     double num = 0.0, den = 0.0;
     for (int n = 1; n <= N; ++n) {
       den = std::fmax(den, hnorms[2 * n]);
