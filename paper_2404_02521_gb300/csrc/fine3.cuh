@@ -21,6 +21,7 @@ struct F3Item {
   float* b;    // [M^3] dtau R_h u of the step
   float* dA;   // [M^3] increment ping-pong
   float* dB;
+  float* dP;   // [M^3] the previous step's increment
   float tau0;
 };
 
