@@ -48,20 +48,12 @@ struct SweepParams {
   float4 rowc[kMaxBandRows];
 };
 
-// BiCGSTAB scalar state shared by a CTA (identical in every CTA of the cluster).  The
-// Krylov dot products and scalars are FP32 like the vectors; only the Parareal norms are
-// FP64 (tot), since FP64 arithmetic runs at a small fraction of the FP32 rate on this GPU
-// and sits on the serial path of every iteration.
+// FP64 totals of the last cluster_sum, shared by a CTA (the Parareal norms; the Krylov scalars
+// are FP32 and live in registers, since FP64 arithmetic runs at a small fraction of the FP32
+// rate on this GPU and would sit on the serial path of every iteration).
 struct Scal {
-  double tot[4];    // FP64 totals of the last cluster_sum<double>
-  float totf[4];    // FP32 totals of the last cluster_sum<float>
-  float rho, alpha, omega, stop2;
-  float af, of, bf;
-  int conv, fail;
+  double tot[4];
 };
-
-__device__ __forceinline__ double* scal_tot(Scal* s, double) { return s->tot; }
-__device__ __forceinline__ float* scal_tot(Scal* s, float) { return s->totf; }
 
 // Jacobi-scaled operator at one node:
 //   (A^ y)_C = y_C - invd * (ce y_E + cw y_W + cs y_S + cn y_N + cg ((y_SE - y_NE) - (y_SW - y_NW)))
@@ -123,7 +115,7 @@ __device__ __forceinline__ T warp_butterfly(T x) {
 // butterfly; warp 0 adds the warp partials (wpart) and lanes 0..C-1 store the CTA partial into
 // slot `rank` of every CTA of the cluster; after one cluster barrier, thread 0 of every CTA
 // adds the C partials in rank order, so every CTA gets bitwise the same totals in
-// scal_tot(sc) (type T), and runs `fin(sc)` before the closing CTA barrier.  `round`
+// sc->tot, and runs `fin(sc)` before the closing CTA barrier.  `round`
 // alternates two slot arrays so that a fast CTA never overwrites partials that a slow CTA is
 // still adding.  slots: double[2][kMaxCluster][4]; wpart: double[NW][4].
 template <class CFG, int NV, class T, class Fin>
@@ -153,7 +145,7 @@ __device__ __forceinline__ void cluster_sum(cg::cluster_group& cl, const T (&v)[
   }
   if (C > 1) cl.sync(); else __syncthreads();
   if (threadIdx.x == 0) {
-    T* out = scal_tot(sc, T(0));
+    T* out = sc->tot;
 #pragma unroll
     for (int q = 0; q < NV; ++q) {
       T acc = T(0);
@@ -165,34 +157,6 @@ __device__ __forceinline__ void cluster_sum(cg::cluster_group& cl, const T (&v)[
   __syncthreads();
   ++round;
 }
-
-// BiCGSTAB scalar updates shared by the band and global kernels (run by one thread per CTA).
-struct KrylovFin {
-  // start: totf = {(b^, b^), (r, r)}
-  static __device__ __forceinline__ void start(Scal* s, float tol) {
-    s->rho = s->totf[1];
-    s->stop2 = tol * tol * s->totf[0];
-    s->conv = s->totf[1] <= s->stop2 || !(s->totf[0] > 1e-30f);
-    s->fail = 0;
-    s->alpha = s->omega = 1.f;
-  }
-  // after v = A^ p: totf = {(r^, v), (r, r)}
-  static __device__ __forceinline__ void alpha(Scal* s) {
-    if (s->totf[1] <= s->stop2) { s->conv = 1; return; }
-    if (s->totf[0] == 0.f) { s->fail = 1; return; }
-    s->alpha = s->rho / s->totf[0];
-    s->af = s->alpha;
-  }
-  // after t = A^ s: totf = {(t, s), (t, t), (r^, s), (r^, t)}
-  static __device__ __forceinline__ void omega(Scal* s) {
-    s->omega = s->totf[1] > 0.f ? s->totf[0] / s->totf[1] : 0.f;
-    s->of = s->omega;
-    const float rho_new = s->totf[2] - s->omega * s->totf[3];
-    if (s->omega == 0.f || s->rho == 0.f) { s->fail = 1; s->bf = 0.f; return; }
-    s->bf = (rho_new / s->rho) * (s->alpha / s->omega);
-    s->rho = rho_new;
-  }
-};
 
 // ---------------------------------------------------------------------------------------
 // Point-to-point cluster exchange for the BiCGSTAB iterations.  A round moves every CTA's
@@ -958,418 +922,6 @@ static int launch_sweep_k(const SweepParams& sp, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------------------------------
-// Grids beyond one cluster's shared memory (M > 256): the same BiCGSTAB and Parareal sweep
-// with the vectors in a global workspace.  One cluster of CG CTAs owns the system; CTA rank
-// handles rows [rank*BHg, rank*BHg + BHg).  Each stencil pass stages its operand rows (R rows
-// of the band plus one halo row on each side) in shared memory once, so every value crosses
-// L2 once rather than nine times; the rows written by other CTAs are read with ld.global.cg
-// (L2, never a stale L1 line), ordered by the cluster barrier's release/acquire.
-// ---------------------------------------------------------------------------------------
-constexpr int kGThreads = 1024;
-struct GCfg {
-  static constexpr int NW = kGThreads / 32;
-};
-
-struct GlobalVecs {
-  float *u, *x, *xp, *xq, *r, *rh, *p, *v, *s, *t, *id, *q;   // q: M^{-1} p, then M^{-1} s
-};
-constexpr int kGlobalVecs = 12;
-
-struct GSweepParams {
-  ItemDesc d;
-  SweepArgs a;
-  GlobalVecs w;
-  int M, C;
-  float h;
-};
-
-__device__ __forceinline__ void g_coefs(const ItemDesc& d, int i, int j, float& ce, float& cw,
-                                        float& cs, float& cn, float& cg) {
-  float cgi, gj;
-  column_coefs(d, i, ce, cw, cgi);
-  row_coefs(d, j, cs, cn, gj);
-  cg = cgi * gj;
-}
-
-// Shared-memory tiles of the stencil passes: rows ra-1 .. rb of an M-column vector with row
-// stride S = M + 8; column c sits at index c + 4, so columns -1 and M read the zero pads and
-// 16-byte copies land aligned.  Rows outside the grid are zero.
-constexpr int kTilePad = 4;
-__host__ __device__ inline int g_tile_stride(int M) { return M + 2 * kTilePad; }
-
-__device__ __forceinline__ void g_stage(const float* __restrict__ y, float* __restrict__ tile, int M, int ra, int rb) {
-  const int S = g_tile_stride(M);
-  const int rows = rb - ra + 2;   // ra-1 .. rb
-  if ((M & 3) == 0) {
-    const int q = M >> 2;
-#pragma unroll 4
-    for (int idx = threadIdx.x; idx < rows * q; idx += kGThreads) {
-      const int r = idx / q, c4 = idx - r * q;
-      const int j = ra - 1 + r;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (j >= 0 && j < M) v = __ldcg(reinterpret_cast<const float4*>(y + (size_t)j * M) + c4);
-      *reinterpret_cast<float4*>(tile + r * S + kTilePad + 4 * c4) = v;
-    }
-  } else {
-#pragma unroll 4
-    for (int idx = threadIdx.x; idx < rows * M; idx += kGThreads) {
-      const int r = idx / M, c = idx - r * M;
-      const int j = ra - 1 + r;
-      tile[r * S + kTilePad + c] = (j >= 0 && j < M) ? __ldcg(y + (size_t)j * M + c) : 0.f;
-    }
-  }
-}
-
-// A^ y at node (i, j) from a tile whose first row is ra - 1.
-__device__ __forceinline__ float g_tile_matvec(const float* tile, int S, int ra, int i, int j, float id, float ce,
-                                               float cw, float cs, float cn, float cg) {
-  const float* c = tile + (j - ra + 1) * S + kTilePad + i;
-  const float yc = c[0], yw = c[-1], ye = c[1];
-  const float yn = c[-S], ys = c[S], ynw = c[-S - 1], yne = c[-S + 1], ysw = c[S - 1], yse = c[S + 1];
-  return yc - id * (ce * ye + cw * yw + cs * ys + cn * yn + cg * ((yse - yne) - (ysw - ynw)));
-}
-
-// Rows of a band per staged pass: two tiles of R + 2 rows in the dynamic shared memory.
-__host__ __device__ inline int g_tile_rows(int M, int BHg, size_t smem_bytes) {
-  const int fit = (int)(smem_bytes / (2 * sizeof(float) * (size_t)g_tile_stride(M))) - 2;
-  return fit < BHg ? (fit > 0 ? fit : 1) : BHg;
-}
-constexpr size_t kGTileBytes = 200 * 1024;   // dynamic shared memory of the global sweep
-
-// Visits the nodes e = b0 + tid, b0 + tid + kGThreads, ... < b1 as f(e, i, j), stepping (i, j)
-// instead of dividing e by M at every node (a 64-bit division is a long instruction sequence).
-template <class F>
-__device__ __forceinline__ void g_nodes(size_t b0, size_t b1, int M, F f) {
-  const int step_j = kGThreads / M, step_i = kGThreads - step_j * M;
-  size_t e = b0 + threadIdx.x;
-  int j = (int)(e / (size_t)M), i = (int)(e - (size_t)j * M);
-  for (; e < b1; e += kGThreads) {
-    f(e, i, j);
-    i += step_i;
-    j += step_j;
-    if (i >= M) {
-      i -= M;
-      ++j;
-    }
-  }
-}
-
-// One stencil pass over the CTA's rows j0..j1-1: stage y0 (and y1) tile by tile, then run
-// body(e, i, j, ra) for every node of the tile's rows (ra: the tile's first own row).
-template <class Body>
-__device__ __forceinline__ void g_pass(const float* y0, const float* y1, float* t0, float* t1, int M, int j0, int j1,
-                                       int R, Body body) {
-  for (int ra = j0; ra < j1; ra += R) {
-    const int rb = min(j1, ra + R);
-    g_stage(y0, t0, M, ra, rb);
-    if (y1) g_stage(y1, t1, M, ra, rb);
-    __syncthreads();
-    g_nodes((size_t)ra * M, (size_t)rb * M, M, [&](size_t e, int i, int j) { body(e, i, j, ra); });
-    __syncthreads();   // the tiles are restaged next
-  }
-}
-
-__global__ void __launch_bounds__(kGThreads, 1) sweep_global_kernel(const __grid_constant__ GSweepParams gp) {
-  cg::cluster_group cluster = cg::this_cluster();
-  const ItemDesc& d = gp.d;
-  const SweepArgs& a = gp.a;
-  const bool batched = a.mode == SWEEP_PROP && a.nprop > 0;
-  const PropItem pit = batched ? a.prop[blockIdx.y] : PropItem{a.in, a.out, d.tau0};
-  // per-state workspace of a batched PROP launch
-  GlobalVecs w = gp.w;
-  if (batched) {
-    const size_t off = (size_t)blockIdx.y * kGlobalVecs * (size_t)gp.M * gp.M;
-    w.u += off; w.x += off; w.xp += off; w.xq += off; w.r += off; w.rh += off;
-    w.p += off; w.v += off; w.s += off; w.t += off; w.id += off; w.q += off;
-  }
-  const int M = gp.M, C = gp.C;
-  const int rank = C > 1 ? (int)cluster.block_rank() : 0;
-  const int tid = threadIdx.x;
-  const size_t MM = (size_t)M * M;
-  const int BHg = (M + C - 1) / C;
-  const int j0 = rank * BHg, j1 = min(M, j0 + BHg);
-  const size_t e0 = (size_t)j0 * M, e1 = (size_t)j1 * M;
-  const PayoffF pf = make_payoff(d);
-  const float rdt = d.rdt;
-  const float tol = (float)a.tol;
-  __shared__ double slots[2 * kMaxCluster * 4];
-  __shared__ double wpart[GCfg::NW * 4];
-  __shared__ Scal scs;
-  Scal* sc = &scs;
-  extern __shared__ __align__(16) float gtiles[];
-  const int S = g_tile_stride(M);
-  const int R = g_tile_rows(M, BHg, kGTileBytes);
-  float* T0 = gtiles;
-  float* T1 = gtiles + (R + 2) * S;
-  for (int idx = tid; idx < 2 * (R + 2) * S; idx += kGThreads) gtiles[idx] = 0.f;   // pads stay zero
-  int round = 0, iters_max = 0, iters_total = 0, nsolves = 0, nhist = 0;
-  bool failed = false;
-  auto barrier = [&]() { __threadfence(); cluster_barrier(cluster, C); };
-
-  const int n_lo = a.n_end > 0 ? a.n_begin : a.n_first;
-  const int n_hi = a.n_end > 0 ? a.n_end : (a.mode == SWEEP_PROP ? a.n_first + 1 : a.N);
-  g_nodes(e0, e1, M, [&](size_t e, int i, int j) {
-    w.id[e] = (i < M - 1 && j < M - 1) ? inv_diag(d, i, j) : 0.f;
-    w.x[e] = 0.f;
-    w.xp[e] = 0.f;
-    w.xq[e] = 0.f;
-    w.q[e] = 0.f;
-    const float* src = a.mode == SWEEP_PROP   ? pit.in
-                       : a.mode == SWEEP_INIT ? a.U + (size_t)n_lo * MM
-                       : n_lo == a.n_first    ? a.Gold + (size_t)a.n_first * MM
-                                              : a.U + (size_t)n_lo * MM;
-    w.u[e] = src[e];
-  });
-  barrier();
-  for (int n = n_lo; n < n_hi; ++n) {
-    const bool skip_g = (a.mode == SWEEP_ITER && n == a.n_first);
-    if (!skip_g) {
-      for (int cstep = 0; cstep < a.csteps; ++cstep) {
-        const float tau_new = (float)(pit.tau0 + a.slice_len * n + (cstep + 1) * d.dtau);
-        // initial guess 3 d_{m-1} - 3 d_{m-2} + d_{m-3} (see the band kernel); x holds d_{m-1}
-        g_nodes(e0, e1, M, [&](size_t e, int i, int j) {
-          if (i == M - 1 || j == M - 1) w.u[e] = far_field(pf, i * gp.h, j * gp.h, tau_new);
-          const float d1 = w.x[e], d2 = w.xp[e];
-          if (nhist >= 3) w.x[e] = 3.f * (d1 - d2) + w.xq[e];
-          else if (nhist == 2) w.x[e] = 2.f * d1 - d2;
-          w.xq[e] = d2;
-          w.xp[e] = d1;
-        });
-        barrier();
-        int it = 0;
-        // restart from the current iterate after a breakdown (see the band kernel)
-        for (int attempt = 0; attempt < kKrylovAttempts; ++attempt) {
-          if (attempt > 0) barrier();   // the other CTAs' last x updates are visible
-          // b^ = D^{-1} dtau R_h w ;  r = b^ - A^ x (x = previous increment)
-          float part[2] = {0.f, 0.f};
-          g_pass(w.u, w.x, T0, T1, M, j0, j1, R, [&](size_t e, int i, int j, int ra) {
-            float bh = 0.f, rr = 0.f;
-            if (i < M - 1 && j < M - 1) {
-              float ce, cw, cs, cn, cg;
-              g_coefs(d, i, j, ce, cw, cs, cn, cg);
-              const float* y = T0 + (j - ra + 1) * S + kTilePad + i;
-              const float c = y[0], yw = y[-1], ye = y[1], yn = y[-S], ys = y[S];
-              const float ynw = y[-S - 1], yne = y[-S + 1], ysw = y[S - 1], yse = y[S + 1];
-              const float b = ce * (ye - c) - cw * (c - yw) + cs * (ys - c) - cn * (c - yn) +
-                              cg * ((yse - yne) - (ysw - ynw)) - rdt * c;
-              const float id = w.id[e];
-              bh = b * id;
-              rr = bh - g_tile_matvec(T1, S, ra, i, j, id, ce, cw, cs, cn, cg);
-            }
-            w.r[e] = rr;
-            w.rh[e] = rr;
-            part[0] = fmaf(bh, bh, part[0]);
-            part[1] = fmaf(rr, rr, part[1]);
-          });
-          cluster_sum<GCfg, 2>(cluster, part, slots, wpart, sc, round, rank, C,
-                               [tol](Scal* s) { KrylovFin::start(s, tol); });
-          for (size_t e = e0 + tid; e < e1; e += kGThreads) w.p[e] = w.r[e];
-          barrier();
-          // Right-preconditioned with M^{-1} = 2I - A^ (see the band kernel): v = A^ M^{-1} p,
-          // t = A^ M^{-1} s, x += alpha M^{-1} p + omega M^{-1} s.  Each preconditioner
-          // application reads its operand's neighbours, hence one more barrier before the
-          // product that reads q.
-          while (!sc->conv && it < a.maxit) {
-            ++it;
-            g_pass(w.p, nullptr, T0, T1, M, j0, j1, R, [&](size_t e, int i, int j, int ra) {
-              float qv = 0.f;
-              if (i < M - 1 && j < M - 1) {
-                float ce, cw, cs, cn, cg;
-                g_coefs(d, i, j, ce, cw, cs, cn, cg);
-                qv = fmaf(2.f, T0[(j - ra + 1) * S + kTilePad + i],
-                          -g_tile_matvec(T0, S, ra, i, j, w.id[e], ce, cw, cs, cn, cg));
-              }
-              w.q[e] = qv;
-            });
-            barrier();
-            float p1[2] = {0.f, 0.f};
-            g_pass(w.q, nullptr, T0, T1, M, j0, j1, R, [&](size_t e, int i, int j, int ra) {
-              float vv = 0.f;
-              if (i < M - 1 && j < M - 1) {
-                float ce, cw, cs, cn, cg;
-                g_coefs(d, i, j, ce, cw, cs, cn, cg);
-                vv = g_tile_matvec(T0, S, ra, i, j, w.id[e], ce, cw, cs, cn, cg);
-              }
-              w.v[e] = vv;
-              const float rr = w.r[e];
-              p1[0] = fmaf(w.rh[e], vv, p1[0]);
-              p1[1] = fmaf(rr, rr, p1[1]);
-            });
-            // every CTA has read its neighbours' q before this reduction's barrier
-            cluster_sum<GCfg, 2>(cluster, p1, slots, wpart, sc, round, rank, C, [](Scal* s) { KrylovFin::alpha(s); });
-            if (sc->conv || sc->fail) break;
-            const float af = sc->af;
-            for (size_t e = e0 + tid; e < e1; e += kGThreads) {
-              w.x[e] = fmaf(af, w.q[e], w.x[e]);
-              w.s[e] = fmaf(-af, w.v[e], w.r[e]);
-            }
-            barrier();
-            g_pass(w.s, nullptr, T0, T1, M, j0, j1, R, [&](size_t e, int i, int j, int ra) {
-              float qv = 0.f;
-              if (i < M - 1 && j < M - 1) {
-                float ce, cw, cs, cn, cg;
-                g_coefs(d, i, j, ce, cw, cs, cn, cg);
-                qv = fmaf(2.f, T0[(j - ra + 1) * S + kTilePad + i],
-                          -g_tile_matvec(T0, S, ra, i, j, w.id[e], ce, cw, cs, cn, cg));
-              }
-              w.q[e] = qv;
-            });
-            barrier();
-            float p2[4] = {0.f, 0.f, 0.f, 0.f};
-            g_pass(w.q, nullptr, T0, T1, M, j0, j1, R, [&](size_t e, int i, int j, int ra) {
-              float tt = 0.f;
-              if (i < M - 1 && j < M - 1) {
-                float ce, cw, cs, cn, cg;
-                g_coefs(d, i, j, ce, cw, cs, cn, cg);
-                tt = g_tile_matvec(T0, S, ra, i, j, w.id[e], ce, cw, cs, cn, cg);
-              }
-              w.t[e] = tt;
-              const float sv = w.s[e], rh = w.rh[e];
-              p2[0] = fmaf(tt, sv, p2[0]);
-              p2[1] = fmaf(tt, tt, p2[1]);
-              p2[2] = fmaf(rh, sv, p2[2]);
-              p2[3] = fmaf(rh, tt, p2[3]);
-            });
-            cluster_sum<GCfg, 4>(cluster, p2, slots, wpart, sc, round, rank, C, [](Scal* s) { KrylovFin::omega(s); });
-            const float of = sc->of, bf = sc->bf;
-            for (size_t e = e0 + tid; e < e1; e += kGThreads) {
-              const float sv = w.s[e], pv = w.p[e], tt = w.t[e];
-              w.x[e] = fmaf(of, w.q[e], w.x[e]);
-              const float rr = fmaf(-of, tt, sv);
-              w.r[e] = rr;
-              w.p[e] = fmaf(bf, fmaf(-of, w.v[e], pv), rr);
-            }
-            if (sc->fail) break;
-            barrier();
-          }
-          if (sc->conv || !sc->fail) break;
-        }
-        if (!sc->conv) failed = true;
-        iters_max = it > iters_max ? it : iters_max;
-        iters_total += it;
-        ++nsolves;
-        nhist = nhist < 3 ? nhist + 1 : 3;
-        for (size_t e = e0 + tid; e < e1; e += kGThreads) w.u[e] += w.x[e];
-        barrier();
-      }
-    }
-    if (a.mode == SWEEP_PROP) {
-      for (size_t e = e0 + tid; e < e1; e += kGThreads) pit.out[e] = w.u[e];
-    } else {
-      double nr[2] = {0.0, 0.0};
-      float* Un = a.U + (size_t)(n + 1) * MM;
-      const float* Fn = a.Fb + (size_t)n * MM;
-      float* Gn = a.Gold + (size_t)n * MM;
-      for (size_t e = e0 + tid; e < e1; e += kGThreads) {
-        const float gnew = w.u[e];
-        // squares in FP32 (u_new - u_old of nearby values is exact), sums in FP64
-        if (a.mode == SWEEP_INIT) {
-          Un[e] = gnew;
-          Gn[e] = gnew;
-          nr[0] += (double)(gnew * gnew);
-        } else {
-          const float unew = Fn[e] + (gnew - Gn[e]);
-          const float du = unew - Un[e];
-          Un[e] = unew;
-          Gn[e] = gnew;
-          w.u[e] = unew;
-          nr[0] += (double)(unew * unew);
-          nr[1] += (double)(du * du);
-        }
-      }
-      double* norms = a.norms;
-      const int slot_n = n + 1;
-      const bool iter = a.mode == SWEEP_ITER;
-      cluster_sum<GCfg, 2>(cluster, nr, slots, wpart, sc, round, rank, C, [norms, slot_n, rank, iter](Scal* s) {
-        if (rank == 0) { norms[2 * slot_n] = s->tot[0]; norms[2 * slot_n + 1] = iter ? s->tot[1] : 0.0; }
-      });
-      barrier();
-    }
-  }
-  if (rank == 0 && tid == 0) {
-    if (failed) atomicOr(a.status, 1);
-    atomicMax(a.status + 1, iters_max);
-    atomicAdd(a.status + 2, iters_total);
-    atomicAdd(a.status + 3, nsolves);
-    if (a.mode == SWEEP_ITER && n_hi == a.N) {
-      double num = 0.0, den = 0.0;
-      for (int n = 1; n <= a.N; ++n) {
-        den = fmax(den, a.norms[2 * n]);
-        if (n >= a.n_first + 1) num = fmax(num, a.norms[2 * n + 1]);
-      }
-      a.defect[0] = den > 0.0 ? sqrt(num) / sqrt(den) : sqrt(num);
-    }
-  }
-}
-
-static cudaLaunchConfig_t global_launch_config(int C, int nst, cudaStream_t s, cudaLaunchAttribute (&attr)[1]) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(C, nst, 1);
-  cfg.blockDim = dim3(kGThreads, 1, 1);
-  cfg.dynamicSmemBytes = kGTileBytes;
-  cfg.stream = s;
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = C;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cfg;
-}
-
-// Cluster size of the global-memory sweep: 16 CTAs where the device can hold such a cluster,
-// else 8 (0: neither).
-static int global_cluster_ctas(int) {
-  if (cudaFuncSetAttribute(sweep_global_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGTileBytes) !=
-      cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  for (int C : {16, 8}) {
-    if (C > 8 &&
-        cudaFuncSetAttribute(sweep_global_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-      cudaGetLastError();
-      continue;
-    }
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = global_launch_config(C, 1, nullptr, attr);
-    int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, sweep_global_kernel, &cfg) != cudaSuccess || nclusters < 1) {
-      cudaGetLastError();
-      continue;
-    }
-    return C;
-  }
-  return 0;
-}
-
-static int launch_sweep_global(const bs_grid* g, const ItemDesc& d, const SweepArgs& a, cudaStream_t s) {
-  const int M = g->M;
-  const size_t MM = (size_t)M * M;
-  const int nst = a.mode == SWEEP_PROP && a.nprop > 0 ? a.nprop : 1;
-  int rc = ensure(const_cast<bs_grid*>(g)->ws_coarse, (size_t)nst * kGlobalVecs * MM * sizeof(float));
-  if (rc) return rc;
-  GSweepParams gp;
-  gp.d = d;
-  gp.a = a;
-  float* base = (float*)g->ws_coarse.ptr;
-  gp.w = GlobalVecs{base,          base + MM,     base + 2 * MM, base + 3 * MM, base + 4 * MM,  base + 5 * MM,
-                    base + 6 * MM, base + 7 * MM, base + 8 * MM, base + 9 * MM, base + 10 * MM, base + 11 * MM};
-  gp.M = M;
-  gp.h = (float)(g->xmax / (M - 1));
-  const int C = global_cluster_ctas(M);
-  if (C == 0) return set_error(BS_ERR_CUDA, "coarse propagator: no cluster shape available for M=%d", M);
-  const int R = g_tile_rows(M, (M + C - 1) / C, kGTileBytes);
-  if ((size_t)2 * (R + 2) * g_tile_stride(M) * sizeof(float) > kGTileBytes)
-    return set_error(BS_ERR_ARG, "coarse propagator: M=%d exceeds the global solver's tile size", M);
-  gp.C = C;
-  cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = global_launch_config(C, nst, s, attr);
-  BS_CUDA_TRY(cudaLaunchKernelEx(&cfg, sweep_global_kernel, gp));
-  return BS_OK;
-}
-
-// ---------------------------------------------------------------------------------------
 // Band variants of the cluster-resident coarse sweep.  A variant fixes the columns per CTA
 // (NCOL >= M), the threads per CTA and the rows per thread; its cluster size follows from M.
 // More CTAs per system shorten the arithmetic of each BiCGSTAB iteration but not its cluster
@@ -1617,7 +1169,7 @@ int coarse_variant_info(int v, int M, int* ctas, int* threads, int* rows, int* p
 
 int coarse_cluster_ctas(const bs_grid* g, const ItemDesc& d, cudaStream_t s, int* ctas) {
   if (variant_ncol(g->M) == 0) {
-    *ctas = global_cluster_ctas(g->M);
+    *ctas = 0;   // beyond one cluster: the grid solver
     return BS_OK;
   }
   int v = -1;
@@ -1633,7 +1185,7 @@ int launch_sweep(const bs_grid* g, const ItemDesc& d, const SweepArgs& a, cudaSt
   sp.a = a;
   sp.sh = g->shape;
   sp.h = (float)(g->xmax / (g->M - 1));
-  if (variant_ncol(g->M) == 0) return launch_sweep_global(g, d, a, s);
+  if (variant_ncol(g->M) == 0) return launch_sweep_grid(g, d, a, s);   // beyond one cluster
   int v = -1;
   int rc = resolve_variant(g, d, s, &v);
   if (rc) return rc;

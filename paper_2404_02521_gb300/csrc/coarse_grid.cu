@@ -1,0 +1,539 @@
+// Numerical coarse propagator G and the serial Parareal sweep on grids beyond one cluster's shared
+// memory (M > 256): the solver of coarse.cu (BiCGSTAB on the Jacobi-scaled system, right
+// preconditioned with M^{-1} = 2I - A^, extrapolated first guesses) with its vectors in a global
+// workspace, one cooperative launch per call.
+//
+// A state is owned by a group of blocks, one tile of kCgW x kCgH nodes per block where the GPU
+// holds that many blocks, else several.  An iteration is two passes over the group's tiles, each
+// followed by one barrier of the group that also carries its dot products:
+//   A  x += omega M^{-1} s, r = s - omega t, p = r + beta (p - omega v), v = A^ M^{-1} p:
+//      (r^, v), (r, r)
+//   B  x += alpha M^{-1} p, s = r - alpha v, t = A^ M^{-1} s: (t, s), (t, t), (r^, s), (r^, t)
+// A pass stages its operand (p or s) in shared memory with two halo rows and columns, forming it
+// from the vectors that its owners wrote before the last barrier, evaluates M^{-1} of it on the
+// tile and one halo row and column, and then the product; nothing is exchanged in between.
+// p and v alternate between two buffers, because a neighbour may still read the old ones.
+//
+// What bounds it: two barriers, two rounds of L2 loads and the latency of short passes per
+// iteration, 10.6 us at 512 x 512 on 128 blocks (49.5 us in the former layout, one cluster of 16
+// SMs with eight cluster barriers and every vector update through L2).  64 x 32 tiles keep a
+// 512 x 512 state's vectors in the registers of one block per tile (12% of the staged nodes
+// are halo); up to 304 tiles are resident, above that (about 780 x 780) a block passes its
+// tiles through the workspace (1024 x 1024: 29.5 us per iteration, 172 before).  States of a batched
+// launch run side by side in as many groups of blocks as the GPU holds, then one after
+// another (10 states of 301 x 301: 2.5 us per iteration, 7.0 before).
+#include <algorithm>
+#include <mutex>
+
+#include "common.cuh"
+#include "grid_barrier.cuh"
+
+namespace bsp {
+
+constexpr int kCgThreads = 256;
+constexpr int kCgW = 64, kCgH = 32;                 // nodes of a tile
+constexpr int kCgK = kCgW * kCgH / kCgThreads;      // nodes of a thread: a strip of one column
+constexpr int kCgS = kCgW + 4;                      // row length of the staged operands: two halo columns
+constexpr int kCgHalo = 2 * 2 * kCgS + 2 * 2 * kCgH;          // nodes of an operand's halo
+constexpr int kCgRing = 2 * (kCgW + 2) + 2 * kCgH;            // nodes of its inner ring
+constexpr int kCgAttempts = 3;                      // BiCGSTAB starts per implicit step
+constexpr int kCgVectors = 13;
+
+struct CgArgs {
+  ItemDesc d;        // dtau = coarse step
+  SweepArgs a;
+  float* ws;         // per group: kCgVectors vectors of M*M
+  GridWords* words;  // per group, zero at launch
+  double2* npart;    // per group: [2][kGridMaxBlocks] (norms)
+  int M, group_blocks, groups;
+  float h;
+};
+
+// weighted neighbours of the entry y of a staged operand
+__device__ __forceinline__ float cg_off(const float* y, float ce, float cw, float cs, float cn, float cg) {
+  return ce * y[1] + cw * y[-1] + cs * y[kCgS] + cn * y[-kCgS] +
+         cg * ((y[kCgS + 1] - y[-kCgS + 1]) - (y[kCgS - 1] - y[-kCgS - 1]));
+}
+
+// ONE: every block owns one tile, whose Krylov vectors stay in registers; only the nodes that a
+// neighbour stages (two rows and columns along the tile's edges) are written to the workspace.
+// Otherwise a pass loads and stores them tile by tile.
+template <bool ONE>
+__global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(const __grid_constant__ CgArgs ca) {
+  constexpr int K = kCgK;
+  const ItemDesc& d = ca.d;
+  const SweepArgs& a = ca.a;
+  const int M = ca.M, tid = threadIdx.x;
+  const size_t MM = (size_t)M * M;
+  const int group = blockIdx.x / ca.group_blocks;
+  GridGroup<kCgThreads> grid{ca.words + group, a.status,
+                             (int)blockIdx.x % ca.group_blocks, ca.group_blocks, tid};
+  float* w0 = ca.ws + (size_t)group * kCgVectors * MM;
+  float *const gu = w0, *const gx = w0 + MM, *const gxp = w0 + 2 * MM, *const gxq = w0 + 3 * MM, *const gr = w0 + 4 * MM,
+              *const grh = w0 + 5 * MM, *const gs = w0 + 6 * MM, *const gt = w0 + 7 * MM, *const gq = w0 + 8 * MM;
+  float* const gp[2] = {w0 + 9 * MM, w0 + 10 * MM};
+  float* const gv[2] = {w0 + 11 * MM, w0 + 12 * MM};
+  __shared__ float P[kCgS * (kCgH + 4)], Q[kCgS * (kCgH + 4)];
+  const PayoffF pf = make_payoff(d);
+  const float rdt = d.rdt, tol = (float)a.tol;
+  const int tiles_i = (M + kCgW - 1) / kCgW, tiles = tiles_i * ((M + kCgH - 1) / kCgH);
+  const int tc = tid % kCgW, r0 = tid / kCgW * K;   // the thread's column and first row of a tile
+  const int L0 = (r0 + 2) * kCgS + tc + 2;          // and its index in P and Q
+  int i0 = 0, j0 = 0;
+  float ce = 0.f, cw = 0.f, cgi = 0.f, id[K];       // of the current tile's strip; id is 0 off the PDE rows
+
+  auto enter = [&](int tile) {
+    j0 = tile / tiles_i * kCgH;
+    i0 = tile % tiles_i * kCgW;
+    const int i = i0 + tc;
+    column_coefs(d, i, ce, cw, cgi);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int j = j0 + r0 + k;
+      id[k] = i < M - 1 && j < M - 1 ? inv_diag(d, i, j) : 0.f;
+    }
+  };
+  auto each_tile = [&](auto&& body) {
+    if constexpr (ONE) {
+      body();
+    } else {
+      for (int tile = grid.block; tile < tiles; tile += grid.blocks) {
+        enter(tile);
+        body();
+        __syncthreads();   // the staged operands are rewritten
+      }
+    }
+  };
+  if constexpr (ONE) enter(grid.block);
+  // f(k, e) for the nodes of the strip that lie in the grid, e their index
+  auto strip = [&](auto&& f) {
+    const int i = i0 + tc;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int j = j0 + r0 + k;
+      if (i < M && j < M) f(k, (size_t)j * M + i);
+    }
+  };
+  auto load = [&](const float* g, float (&v)[K]) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) v[k] = 0.f;
+    strip([&](int k, size_t e) { v[k] = g[e]; });
+  };
+  auto store = [&](float* g, const float (&v)[K]) { strip([&](int k, size_t e) { g[e] = v[k]; }); };
+  // what a neighbour stages (ONE) or the next pass loads
+  auto share = [&](float* g, const float (&v)[K]) {
+    strip([&](int k, size_t e) {
+      if (!ONE || tc < 2 || tc >= kCgW - 2 || r0 + k < 2 || r0 + k >= kCgH - 2) g[e] = v[k];
+    });
+  };
+  // own nodes of an operand into its tile
+  auto put = [&](float* dst, const float (&v)[K]) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) dst[L0 + k * kCgS] = v[k];
+  };
+  // its halo: val(e) inside the grid, zero outside
+  auto halo = [&](float* dst, auto&& val) {
+#pragma unroll
+    for (int n = 0; n < (kCgHalo + kCgThreads - 1) / kCgThreads; ++n) {
+      const int h = tid + n * kCgThreads;
+      if (h >= kCgHalo) break;
+      int row, c;
+      if (h < 4 * kCgS) {
+        const int w = h / kCgS;
+        row = w < 2 ? w : w + kCgH;
+        c = h - w * kCgS;
+      } else {
+        const int w = h - 4 * kCgS;
+        row = 2 + (w >> 2);
+        c = (w & 1) + ((w & 2) ? kCgW + 2 : 0);
+      }
+      const int i = i0 + c - 2, j = j0 + row - 2;
+      dst[row * kCgS + c] = i >= 0 && i < M && j >= 0 && j < M ? val((size_t)j * M + i) : 0.f;
+    }
+  };
+  // f(k, y, A^ y) down the strip, y the operand's nodes
+  auto product = [&](const float* src, auto&& f) {
+    const float* y = src + L0;
+    float nW = y[-kCgS - 1], nC = y[-kCgS], nE = y[-kCgS + 1], cW = y[-1], cC = y[0], cE = y[1];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const float sW = y[(k + 1) * kCgS - 1], sC = y[(k + 1) * kCgS], sE = y[(k + 1) * kCgS + 1];
+      float cs, cn, gj;
+      row_coefs(d, j0 + r0 + k, cs, cn, gj);
+      const float off = ce * cE + cw * cW + cs * sC + cn * nC + cgi * gj * ((sE - nE) - (sW - nW));
+      f(k, cC, cC - id[k] * off);
+      nW = cW; nC = cC; nE = cE;
+      cW = sW; cC = sC; cE = sE;
+    }
+  };
+  // Q = M^{-1} P = 2 P - A^ P on the tile (also in q) and one ring around it, then av = A^ Q
+  auto precond_product = [&](float (&q)[K], float (&av)[K]) {
+    __syncthreads();
+    product(P, [&](int k, float y, float ay) {
+      q[k] = fmaf(2.f, y, -ay);
+      Q[L0 + k * kCgS] = q[k];
+    });
+    if (tid < kCgRing) {
+      int row, c;
+      if (tid < 2 * (kCgW + 2)) {
+        row = tid < kCgW + 2 ? 1 : kCgH + 2;
+        c = 1 + (tid < kCgW + 2 ? tid : tid - (kCgW + 2));
+      } else {
+        const int w = tid - 2 * (kCgW + 2);
+        row = 2 + (w >> 1);
+        c = (w & 1) ? kCgW + 2 : 1;
+      }
+      const int i = i0 + c - 2, j = j0 + row - 2;
+      float val = 0.f;
+      if (i >= 0 && i < M - 1 && j >= 0 && j < M - 1) {
+        float e, w, g, cs, cn, gj;
+        column_coefs(d, i, e, w, g);
+        row_coefs(d, j, cs, cn, gj);
+        const float* y = P + row * kCgS + c;
+        val = fmaf(2.f, y[0], -(y[0] - inv_diag(d, i, j) * cg_off(y, e, w, cs, cn, g * gj)));
+      }
+      Q[row * kCgS + c] = val;
+    }
+    __syncthreads();
+    product(Q, [&](int k, float, float aq) { av[k] = aq; });
+  };
+
+  const bool batched = a.mode == SWEEP_PROP && a.nprop > 0;
+  const int nstates = batched ? a.nprop : 1;
+  const int n_lo = a.n_end > 0 ? a.n_begin : a.n_first;
+  const int n_hi = a.n_end > 0 ? a.n_end : (a.mode == SWEEP_PROP ? a.n_first + 1 : a.N);
+  int iters_max = 0, iters_total = 0, nsolves = 0;
+  bool failed = false;
+  // the strip's x, r (s after an iteration's first pass), r^, p, v, t and M^{-1} p (then M^{-1} s)
+  float x[K], r[K], rh[K], p[K], v[K], t[K], q[K];
+
+  for (int st = group; st < nstates && !grid.dead; st += ca.groups) {
+    const PropItem pit = batched ? a.prop[st] : PropItem{a.in, a.out, d.tau0};
+    const float* src = a.mode == SWEEP_PROP   ? pit.in
+                       : a.mode == SWEEP_INIT ? a.U + (size_t)n_lo * MM
+                       : n_lo == a.n_first    ? a.Gold + (size_t)a.n_first * MM   // G(u_k) unchanged: G_old_k
+                                              : a.U + (size_t)n_lo * MM;
+    each_tile([&] {
+      strip([&](int, size_t e) {
+        gu[e] = src[e];
+        gx[e] = 0.f;
+        gxp[e] = 0.f;
+        gxq[e] = 0.f;
+      });
+    });
+    int nhist = 0;
+    for (int n = n_lo; n < n_hi && !grid.dead; ++n) {
+      const bool skip_g = a.mode == SWEEP_ITER && n == a.n_first;
+      for (int cstep = 0; cstep < (skip_g ? 0 : a.csteps) && !grid.dead; ++cstep) {
+        const float tau_new = (float)(pit.tau0 + a.slice_len * n + (cstep + 1) * d.dtau);
+        // far-field data, and the first guess 3 d_{m-1} - 3 d_{m-2} + d_{m-3} (gx holds d_{m-1})
+        each_tile([&] {
+          strip([&](int k, size_t e) {
+            const int i = i0 + tc, j = j0 + r0 + k;
+            if (i == M - 1 || j == M - 1) gu[e] = far_field(pf, i * ca.h, j * ca.h, tau_new);
+            const float d1 = gx[e], d2 = gxp[e];
+            if (nhist >= 3) gx[e] = 3.f * (d1 - d2) + gxq[e];
+            else if (nhist == 2) gx[e] = 2.f * d1 - d2;
+            gxq[e] = d2;
+            gxp[e] = d1;
+          });
+        });
+        int it = 0;
+        bool conv = false, fail = true;
+        // a breakdown (a zero denominator) restarts from the current iterate
+        for (int attempt = 0; attempt < kCgAttempts && !conv && fail && !grid.dead; ++attempt) {
+          grid.barrier();   // the owners' u and x are visible
+          // b^ = D^{-1} dtau R_h u;  r = r^ = p = b^ - A^ x
+          float sums[4] = {0.f, 0.f, 0.f, 0.f};
+          each_tile([&] {
+            load(gx, x);
+            float u[K], ax[K];
+            load(gu, u);
+            put(P, u);
+            put(Q, x);
+            halo(P, [&](size_t e) { return __ldcg(gu + e); });
+            halo(Q, [&](size_t e) { return __ldcg(gx + e); });
+            __syncthreads();
+            product(Q, [&](int k, float, float ay) { ax[k] = ay; });
+            const float* y = P + L0;
+#pragma unroll
+            for (int k = 0; k < K; ++k, y += kCgS) {
+              float cs, cn, gj;
+              row_coefs(d, j0 + r0 + k, cs, cn, gj);
+              const float c = y[0];
+              const float b = ce * (y[1] - c) - cw * (c - y[-1]) + cs * (y[kCgS] - c) - cn * (c - y[-kCgS]) +
+                              cgi * gj * ((y[kCgS + 1] - y[-kCgS + 1]) - (y[kCgS - 1] - y[-kCgS - 1])) - rdt * c;
+              const float bh = b * id[k];
+              r[k] = rh[k] = p[k] = bh - ax[k];
+              sums[0] = fmaf(bh, bh, sums[0]);
+              sums[1] = fmaf(r[k], r[k], sums[1]);
+            }
+            share(gr, r);
+            share(gp[0], p);
+            if (!ONE) store(grh, rh);
+          });
+          grid.sum(sums);
+          float rho = sums[1];
+          const float stop2 = tol * tol * sums[0];
+          conv = sums[1] <= stop2 || !(sums[0] > 1e-30f);
+          fail = false;
+          float alpha = 0.f, omega = 0.f, beta = 0.f;
+          bool open = false;   // the last iteration's x += omega M^{-1} s is still to be applied
+          for (int m = 0; !conv && !fail && it < a.maxit && !grid.dead; ++m) {
+            ++it;
+            const float *vo = gv[m ? (m - 1) & 1 : 0], *po = gp[m ? (m - 1) & 1 : 0];
+            float *vn = gv[m & 1], *pn = gp[m & 1];
+            float sa[4] = {0.f, 0.f, 0.f, 0.f};
+            each_tile([&] {
+              if (!ONE) {
+                load(grh, rh);
+                load(po, p);
+                if (m == 0) {
+                  load(gr, r);
+                } else {
+                  load(gs, r);
+                  load(gt, t);
+                  load(vo, v);
+                  load(gq, q);
+                  load(gx, x);
+                }
+              }
+              if (m == 0) {   // r and p are at hand
+                halo(P, [&](size_t e) { return __ldcg(po + e); });
+              } else {
+                halo(P, [&](size_t e) {
+                  const float rr = fmaf(-omega, __ldcg(gt + e), __ldcg(gs + e));
+                  return fmaf(beta, fmaf(-omega, __ldcg(vo + e), __ldcg(po + e)), rr);
+                });
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                  x[k] = fmaf(omega, q[k], x[k]);
+                  r[k] = fmaf(-omega, t[k], r[k]);
+                  p[k] = fmaf(beta, fmaf(-omega, v[k], p[k]), r[k]);
+                }
+                share(gr, r);
+                share(pn, p);
+              }
+              put(P, p);
+              precond_product(q, v);
+#pragma unroll
+              for (int k = 0; k < K; ++k) {
+                sa[0] = fmaf(rh[k], v[k], sa[0]);
+                sa[1] = fmaf(r[k], r[k], sa[1]);
+              }
+              share(vn, v);
+              if (!ONE) {
+                store(gq, q);
+                if (m) store(gx, x);
+              }
+            });
+            open = false;
+            grid.sum(sa);
+            if (sa[1] <= stop2) {
+              conv = true;
+              break;
+            }
+            if (sa[0] == 0.f) {
+              fail = true;
+              break;
+            }
+            alpha = rho / sa[0];
+            float sb[4] = {0.f, 0.f, 0.f, 0.f};
+            each_tile([&] {
+              if (!ONE) {
+                load(grh, rh);
+                load(gr, r);
+                load(vn, v);
+                load(gq, q);
+                load(gx, x);
+              }
+              halo(P, [&](size_t e) { return fmaf(-alpha, __ldcg(vn + e), __ldcg(gr + e)); });
+#pragma unroll
+              for (int k = 0; k < K; ++k) {
+                x[k] = fmaf(alpha, q[k], x[k]);
+                r[k] = fmaf(-alpha, v[k], r[k]);
+              }
+              share(gs, r);
+              put(P, r);
+              precond_product(q, t);
+#pragma unroll
+              for (int k = 0; k < K; ++k) {
+                sb[0] = fmaf(t[k], r[k], sb[0]);
+                sb[1] = fmaf(t[k], t[k], sb[1]);
+                sb[2] = fmaf(rh[k], r[k], sb[2]);
+                sb[3] = fmaf(rh[k], t[k], sb[3]);
+              }
+              share(gt, t);
+              if (!ONE) {
+                store(gq, q);
+                store(gx, x);
+              }
+            });
+            grid.sum(sb);
+            open = true;
+            omega = sb[1] > 0.f ? sb[0] / sb[1] : 0.f;
+            const float rho_new = sb[2] - omega * sb[3];
+            if (omega == 0.f || rho == 0.f) {
+              fail = true;
+              beta = 0.f;
+            } else {
+              beta = (rho_new / rho) * (alpha / omega);
+              rho = rho_new;
+            }
+          }
+          each_tile([&] {
+            if (!ONE) {
+              load(gx, x);
+              load(gq, q);
+            }
+            if (open) {
+#pragma unroll
+              for (int k = 0; k < K; ++k) x[k] = fmaf(omega, q[k], x[k]);
+            }
+            store(gx, x);
+          });
+        }
+        if (!conv) failed = true;
+        iters_max = max(iters_max, it);
+        iters_total += it;
+        ++nsolves;
+        nhist = nhist < 3 ? nhist + 1 : 3;
+        each_tile([&] { strip([&](int, size_t e) { gu[e] += gx[e]; }); });
+      }
+      if (a.mode == SWEEP_PROP) {
+        each_tile([&] { strip([&](int, size_t e) { pit.out[e] = gu[e]; }); });
+        continue;
+      }
+      // correction u_{n+1} = F_n + (G_new - G_old_n), squares in FP32 (u_new - u_old of nearby
+      // values is exact), sums in FP64
+      double n0 = 0.0, n1 = 0.0;
+      float* Un = a.U + (size_t)(n + 1) * MM;
+      const float* Fn = a.Fb + (size_t)n * MM;
+      float* Gn = a.Gold + (size_t)n * MM;
+      each_tile([&] {
+        strip([&](int, size_t e) {
+          const float gnew = gu[e];
+          if (a.mode == SWEEP_INIT) {
+            Un[e] = gnew;
+            Gn[e] = gnew;
+            n0 += (double)(gnew * gnew);
+          } else {
+            const float unew = Fn[e] + (gnew - Gn[e]), du = unew - Un[e];
+            Un[e] = unew;
+            Gn[e] = gnew;
+            gu[e] = unew;
+            n0 += (double)(unew * unew);
+            n1 += (double)(du * du);
+          }
+        });
+      });
+      __shared__ double2 wn[kCgThreads / 32];
+      auto reduce = [&](double& b0, double& b1) {   // over the block, the same in all threads
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+          b0 += __shfl_xor_sync(0xffffffffu, b0, off);
+          b1 += __shfl_xor_sync(0xffffffffu, b1, off);
+        }
+        __syncthreads();
+        if ((tid & 31) == 0) wn[tid >> 5] = make_double2(b0, b1);
+        __syncthreads();
+        b0 = b1 = 0.0;
+        for (int w = 0; w < kCgThreads / 32; ++w) {
+          b0 += wn[w].x;
+          b1 += wn[w].y;
+        }
+      };
+      reduce(n0, n1);
+      double2* np = ca.npart + (size_t)group * 2 * kGridMaxBlocks + (n & 1) * kGridMaxBlocks;
+      if (tid == 0) __stcg(np + grid.block, make_double2(n0, n1));
+      grid.barrier();
+      if (grid.block == 0) {   // (the slots alternate by slice: the next slice's barriers order their reuse)
+        n0 = n1 = 0.0;
+        for (int b = tid; b < grid.blocks; b += kCgThreads) {
+          const double2 w = __ldcg(np + b);
+          n0 += w.x;
+          n1 += w.y;
+        }
+        reduce(n0, n1);
+        if (tid == 0) {
+          a.norms[2 * (n + 1)] = n0;
+          a.norms[2 * (n + 1) + 1] = a.mode == SWEEP_ITER ? n1 : 0.0;
+        }
+      }
+    }
+    if (batched && st + ca.groups < nstates) grid.barrier();   // the next state reuses the vectors
+  }
+  if (grid.block == 0 && tid == 0) {
+    if (failed && !grid.dead) atomicOr(a.status, 1);
+    atomicMax(a.status + 1, iters_max);
+    atomicAdd(a.status + 2, iters_total);
+    atomicAdd(a.status + 3, nsolves);
+    if (a.mode == SWEEP_ITER && n_hi == a.N) {
+      double num = 0.0, den = 0.0;
+      for (int n = 1; n <= a.N; ++n) {
+        den = fmax(den, a.norms[2 * n]);
+        if (n >= a.n_first + 1) num = fmax(num, a.norms[2 * n + 1]);
+      }
+      a.defect[0] = den > 0.0 ? sqrt(num) / sqrt(den) : sqrt(num);
+    }
+  }
+}
+
+// Blocks of the solver that the current device runs at once, measured once per device.
+template <bool ONE>
+static int cg_blocks(int* out) {
+  static std::mutex mu;
+  static int known[64] = {};
+  int dev = 0;
+  BS_CUDA_TRY(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lock(mu);
+  int n = dev < 64 ? known[dev] : 0;
+  if (!n) {
+    int per_sm = 0, sms = 0;
+    BS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_grid_kernel<ONE>, kCgThreads, 0));
+    BS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    n = std::min(per_sm * sms, kGridMaxBlocks);
+    if (n < 1) return set_error(BS_ERR_CUDA, "coarse propagator: no block of the grid solver fits an SM");
+    if (dev < 64) known[dev] = n;
+  }
+  *out = n;
+  return BS_OK;
+}
+
+int launch_sweep_grid(const bs_grid* g, const ItemDesc& d, const SweepArgs& a, cudaStream_t s) {
+  const int M = g->M;
+  const size_t MM = (size_t)M * M;
+  const int nst = a.mode == SWEEP_PROP && a.nprop > 0 ? a.nprop : 1;
+  const int tiles = ((M + kCgW - 1) / kCgW) * ((M + kCgH - 1) / kCgH);
+  int blocks = 0;
+  int rc = cg_blocks<true>(&blocks);
+  if (rc) return rc;
+  const bool one = tiles <= blocks;
+  if (!one && (rc = cg_blocks<false>(&blocks))) return rc;
+  CgArgs ca;
+  ca.group_blocks = std::min(tiles, blocks);
+  ca.groups = std::min(nst, blocks / ca.group_blocks);
+  // vectors, the groups' barrier words, norm partials
+  const size_t fbytes = ((size_t)ca.groups * kCgVectors * MM * sizeof(float) + 255) & ~(size_t)255;
+  const size_t pbytes = (size_t)ca.groups * sizeof(GridWords);
+  const size_t nbytes = (size_t)ca.groups * 2 * kGridMaxBlocks * sizeof(double2);
+  rc = ensure(const_cast<bs_grid*>(g)->ws_coarse, fbytes + pbytes + nbytes);
+  if (rc) return rc;
+  unsigned char* ws = static_cast<unsigned char*>(g->ws_coarse.ptr);
+  ca.d = d;
+  ca.a = a;
+  ca.ws = reinterpret_cast<float*>(ws);
+  ca.words = reinterpret_cast<GridWords*>(ws + fbytes);
+  ca.npart = reinterpret_cast<double2*>(ws + fbytes + pbytes);
+  ca.M = M;
+  ca.h = (float)(g->xmax / (M - 1));
+  BS_CUDA_TRY(cudaMemsetAsync(ca.words, 0, pbytes, s));
+  void* args[] = {&ca};
+  void* kern = one ? reinterpret_cast<void*>(sweep_grid_kernel<true>)
+                   : reinterpret_cast<void*>(sweep_grid_kernel<false>);
+  BS_CUDA_TRY(cudaLaunchCooperativeKernel(kern, dim3(ca.group_blocks * ca.groups),
+                                          dim3(kCgThreads), args, 0, s));
+  return BS_OK;
+}
+
+}  // namespace bsp

@@ -295,6 +295,8 @@ struct SweepArgs {
   int n_begin, n_end;
 };
 int launch_sweep(const bs_grid* g, const ItemDesc& d, const SweepArgs& a, cudaStream_t s);
+// ... on grids beyond one cluster (coarse_grid.cu)
+int launch_sweep_grid(const bs_grid* g, const ItemDesc& d, const SweepArgs& a, cudaStream_t s);
 // F by BiCGSTAB per implicit step for items whose Jacobi bound is >= 0.8 (capi.cu)
 int launch_krylov_fine(bs_grid* g, const ItemDesc* items, int n, int nsteps, cudaStream_t s);
 int coarse_cached_variant(int device, int M);   // tuned (or default) variant, no allocation

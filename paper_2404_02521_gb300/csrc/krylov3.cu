@@ -24,93 +24,26 @@
 #include <mutex>
 
 #include "fine3.cuh"
+#include "grid_barrier.cuh"
 
 namespace bsp {
 
 constexpr int kK3Attempts = 3;
 constexpr int kK3Planes = 4;             // planes of k per tile: 256 tiles at 64^3
 constexpr int kK3Threads = kF3TileI * kF3TileJ;
-constexpr int kK3Polls = 1 << 22;        // bound on the polls of one grid barrier
 constexpr int kK3HI = kF3TileI + 2, kK3HJ = kF3TileJ + 2, kK3HK = kK3Planes + 2;
 constexpr int kK3Tile = kK3HI * kK3HJ * kK3HK;
 constexpr int kK3Ring = kK3HI * kK3HJ - kK3Threads;                       // halo entries of an inner plane
 constexpr int kK3Halo = 2 * kK3HI * kK3HJ + kK3Planes * kK3Ring;          // halo entries of a tile
-constexpr int kK3MaxBlocks = 1024;
 
 struct K3Args {
   F3Batch fb;          // item 0: in, out, hi, lo, tau0
   float *x, *r, *rh, *s, *t;
   float *p[2], *v[2];
-  float4* partials;    // [2][kK3MaxBlocks]
-  unsigned* bar;       // arrivals, zero at launch
+  GridWords* words;    // zero at launch
   int* status;         // bit 0: no convergence, bit 1: a barrier timed out; the launch returns at once if set
   int nsteps, maxit;
   float tol;
-};
-
-// Sums over the grid and a barrier: every block returns bitwise the same totals.
-struct K3Grid {
-  const K3Args& a;
-  unsigned target = 0;
-  int round = 0;
-  bool dead = false;
-  __device__ explicit K3Grid(const K3Args& args) : a(args) {}
-
-  __device__ __forceinline__ void barrier() {
-    __shared__ int timeout;
-    if (dead) return;   // the solve is over: leave without another wait
-    target += gridDim.x;
-    __syncthreads();
-    if (threadIdx.x + threadIdx.y == 0) {
-      __threadfence();
-      atomicAdd(a.bar, 1u);
-      int polls = 0, out = 0;
-      unsigned seen = 0;
-      while (true) {
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(seen) : "l"(a.bar) : "memory");
-        if (seen >= target) break;
-        if (++polls >= kK3Polls || ((polls & 1023) == 0 && (*(volatile int*)a.status & 2))) {
-          atomicOr(a.status, 2);
-          out = 1;
-          break;
-        }
-      }
-      timeout = out;
-    }
-    __syncthreads();
-    dead = dead || timeout;
-    __syncthreads();
-  }
-  static __device__ __forceinline__ void block_sum(float (&v)[4], float4* ws) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], off);
-    const int tid = threadIdx.y * kF3TileI + threadIdx.x;
-    if ((tid & 31) == 0) ws[tid >> 5] = make_float4(v[0], v[1], v[2], v[3]);
-    __syncthreads();
-    v[0] = v[1] = v[2] = v[3] = 0.f;
-#pragma unroll
-    for (int w = 0; w < kK3Threads / 32; ++w) {
-      v[0] += ws[w].x; v[1] += ws[w].y; v[2] += ws[w].z; v[3] += ws[w].w;
-    }
-    __syncthreads();
-  }
-  __device__ __forceinline__ void sum(float (&v)[4]) {
-    __shared__ float4 ws[kK3Threads / 32];
-    const int tid = threadIdx.y * kF3TileI + threadIdx.x;
-    float4* slot = a.partials + (round & 1) * kK3MaxBlocks;
-    ++round;
-    block_sum(v, ws);
-    if (tid == 0) __stcg(slot + blockIdx.x, make_float4(v[0], v[1], v[2], v[3]));
-    barrier();
-    v[0] = v[1] = v[2] = v[3] = 0.f;
-    for (int b = tid; b < (int)gridDim.x; b += kK3Threads) {
-      const float4 q = __ldcg(slot + b);
-      v[0] += q.x; v[1] += q.y; v[2] += q.z; v[3] += q.w;
-    }
-    block_sum(v, ws);
-  }
 };
 
 __global__ void __launch_bounds__(kK3Threads, 2) k3_solve_kernel(const __grid_constant__ K3Args a) {
@@ -125,7 +58,7 @@ __global__ void __launch_bounds__(kK3Threads, 2) k3_solve_kernel(const __grid_co
   const int L0 = (kK3HJ + threadIdx.y + 1) * kK3HI + threadIdx.x + 1;   // tile index of the column's first plane
   constexpr int LZ = kK3HI * kK3HJ;
   const F3Coef& c = fb.c;
-  K3Grid grid(a);
+  GridGroup<kK3Threads> grid{a.words, a.status, (int)blockIdx.x, (int)gridDim.x, tid};
 
   int i0 = 0, j0 = 0, k0 = 0;
   // body(kk, e, pde) for every node of the thread's column in this block's tiles, after head()
@@ -387,7 +320,7 @@ static int k3_blocks(int* out) {
     int per_sm = 0, sms = 0;
     BS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k3_solve_kernel, kK3Threads, 0));
     BS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int n = std::min(per_sm * sms, kK3MaxBlocks);
+    const int n = std::min(per_sm * sms, kGridMaxBlocks);
     if (n < 1) return set_error(BS_ERR_CUDA, "three-asset coarse solver: no block fits an SM");
     if (dev >= 64) {
       *out = n;
@@ -402,7 +335,7 @@ static int k3_blocks(int* out) {
 constexpr int kK3Vectors = 11;
 size_t k3_workspace_bytes(int M) {
   const size_t n3 = (size_t)M * M * M;
-  return ((kK3Vectors * n3 * sizeof(float) + 255) & ~(size_t)255) + 2 * kK3MaxBlocks * sizeof(float4) + 256;
+  return ((kK3Vectors * n3 * sizeof(float) + 255) & ~(size_t)255) + sizeof(GridWords) + 256;
 }
 int* k3_status(void* ws, int M) {
   return reinterpret_cast<int*>(static_cast<unsigned char*>(ws) + k3_workspace_bytes(M) - 256);
@@ -429,13 +362,12 @@ int coarse_propagate3_krylov(int M, double xmax, const bs_params3& p, const floa
   float** v[kK3Vectors] = {&it.hi, &it.lo, &a.x, &a.r, &a.rh, &a.s, &a.t, &a.p[0], &a.p[1], &a.v[0], &a.v[1]};
   for (int q = 0; q < kK3Vectors; ++q) *v[q] = f + q * n3;
   a.status = k3_status(ws, M);
-  a.bar = reinterpret_cast<unsigned*>(a.status) + 16;
-  a.partials = reinterpret_cast<float4*>(static_cast<unsigned char*>(ws) + k3_workspace_bytes(M) - 256) - 2 * kK3MaxBlocks;
+  a.words = reinterpret_cast<GridWords*>(reinterpret_cast<unsigned char*>(a.status) - sizeof(GridWords));
   a.nsteps = nsteps;
   a.maxit = maxit;
   a.tol = (float)tol;
   const int tiles = ((M + kF3TileI - 1) / kF3TileI) * ((M + kF3TileJ - 1) / kF3TileJ) * ((M + kK3Planes - 1) / kK3Planes);
-  BS_CUDA_TRY(cudaMemsetAsync(a.bar, 0, sizeof(unsigned), s));
+  BS_CUDA_TRY(cudaMemsetAsync(&a.words->arrivals, 0, sizeof(unsigned), s));
   void* args[] = {&a};
   BS_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(k3_solve_kernel), dim3(std::min(tiles, blocks)),
                                           dim3(kF3TileI, kF3TileJ), args, 0, s));
