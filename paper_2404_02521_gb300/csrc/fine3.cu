@@ -8,7 +8,7 @@
 // second from the previous increment, later ones from the extrapolation of the previous two.  u is
 // carried as a compensated (hi, lo) FP32 pair.  Starting every step from the previous
 // increment took 22 sweeps per step at q = 0.72 (64^3, dtau = 1/640) where the extrapolation
-// takes 13 and, late, 4: 16 states, 40 steps, 24.4 -> 10.4 ms, with the same error against 64
+// takes 13 falling to 4: 16 states, 40 steps, 24.4 -> 9.7 ms, with the same error against 64
 // bits (1.6e-6; 3.6e-6 and 2.2e-6 on longer runs, all unchanged to three digits).
 // Stencil coefficients are products of host-rounded FP32 constants and exact integer node
 // indices (x_p = i_p h, so h cancels).
@@ -222,20 +222,23 @@ double f3_contraction(int M, const bs_params3& p, double dtau) {
   return q;
 }
 
-// Sweeps of step `step` of a propagation, by how its solve starts (as the two-asset stepper):
-// from zero, from the previous increment, from the extrapolation of the previous two, and
-// that after the transients of the start have decayed.  A late count is even: the error
-// recurrence e_{t+1} = l^m (2 e_t - e_{t-1}) of an extrapolated start has a root beyond 1 where
-// l^m < -1/3 (l an eigenvalue of the sweep, which can be negative).
-constexpr int kF3ExtrapStart = 2, kF3ExtrapLate = 16;
+// Sweeps of step `step` of a propagation, by how its solve starts: from zero, from the
+// previous increment, or from the extrapolation of the previous two.  An extrapolated start is
+// off by a mode's second difference in time, and the modes that have survived n steps decay by
+// about 1/n per step, so the reduction that the solve owes falls with n.  A fixed 2^-6 up to
+// step 16 and 1/2 from there takes a tenth fewer sweeps, but on a white-noise state left 6e-6
+// (24^3, q = 0.72, 40 steps) where this leaves the FP32 rounding's 1e-6.  A target above 1/4
+// takes an even count: the error recurrence e_{t+1} = l^m (2 e_t - e_{t-1}) of an extrapolated
+// start has a root beyond 1 where l^m < -1/3 (l an eigenvalue of the sweep, which can be
+// negative).
+constexpr int kF3ExtrapStart = 2;
 static int f3_sweeps(double q, int step) {
   const double target = step == 0               ? 1.0 / 4194304.0
                         : step < kF3ExtrapStart ? 1.0 / 1024.0
-                        : step < kF3ExtrapLate  ? 1.0 / 64.0
-                                                : 0.5;
+                                                : std::fmin(step / 128.0, 0.5);
   if (q <= 0.0) return 2;
   const int m = std::max(2, (int)std::ceil(std::log(target) / std::log(q)));
-  return step < kF3ExtrapLate ? m : (m + 1) & ~1;
+  return target > 0.25 ? (m + 1) & ~1 : m;
 }
 
 int f3_check(int M, double xmax, const bs_params3* p) {
