@@ -6,8 +6,11 @@ library cannot be loaded this module raises, there is no CPU fallback.
 """
 from __future__ import annotations
 
+import array
 import ctypes as C
+import operator
 import os
+import struct
 from typing import Optional, Sequence
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -154,6 +157,51 @@ def to_params(p) -> bs_params:
                      float(getattr(p, "strike2", 0.0)), float(getattr(p, "cash", 1.0)))
 
 
+# bs_params in native layout, and its fields in that order
+_PACK = struct.Struct("8di4x2d")
+_FIELDS = operator.attrgetter("sigma1", "sigma2", "rho", "r", "T", "strike", "w1", "w2", "payoff",
+                              "strike2", "cash")
+assert _PACK.size == C.sizeof(bs_params)
+
+
+def _params_array(params: Sequence, B: int):
+    """bs_params[B] from workloads.Params-like objects, packed into one buffer.  A ctypes
+    structure per item costs three times as much (32 items: 58 us of a call whose kernel takes
+    12), and the slices of one solve repeat an object, which is then packed once."""
+    n = _PACK.size
+    buf = bytearray(n * B)
+    last = None
+    at = 0
+    for p in params:
+        if at == n * B:
+            raise IndexError("more parameter sets than states")
+        if p is last:
+            buf[at:at + n] = buf[at - n:at]
+        else:
+            try:
+                _PACK.pack_into(buf, at, *_FIELDS(p))
+            except (AttributeError, TypeError, struct.error):   # optional fields, other numbers
+                buf[at:at + n] = bytes(to_params(p))
+            last = p
+        at += n
+    return (bs_params * B).from_buffer(buf)
+
+
+def _array(typecode: str, ctype, values: list, B: int):
+    """ctype[B] of `values`; a short list leaves zeros, which the C entry refuses where it has to."""
+    if len(values) > B:
+        raise IndexError("more entries than states")
+    return (ctype * B).from_buffer(array.array(typecode, values + [0] * (B - len(values))))
+
+
+def _pointers(xs: Sequence, B: int):
+    return _array("Q", C.c_void_p, [_ptr(x) for x in xs], B)
+
+
+def _doubles(xs: Sequence, B: int):
+    return _array("d", C.c_double, [float(x) for x in xs], B)
+
+
 def to_params3(p) -> bs_params3:
     """From an object with sigma (3), rho (rho_12, rho_13, rho_23), r, strike, w (3), payoff."""
     return bs_params3((C.c_double * 3)(*[float(v) for v in p.sigma]),
@@ -209,12 +257,8 @@ def fine_propagate_batched(g: Grid, params: Sequence, u_in: Sequence, u_out: Seq
                            tau0: Sequence[float], dtau: Sequence[float], nsteps: int,
                            stream=None):
     B = len(u_in)
-    P = (bs_params * B)(*[to_params(p) for p in params])
-    pin = (C.c_void_p * B)(*[_ptr(x) for x in u_in])
-    pout = (C.c_void_p * B)(*[_ptr(x) for x in u_out])
-    t0 = (C.c_double * B)(*[float(t) for t in tau0])
-    dt = (C.c_double * B)(*[float(t) for t in dtau])
-    return check(load().fine_propagate_batched(g.h, P, pin, pout, t0, dt, int(nsteps), B,
+    return check(load().fine_propagate_batched(g.h, _params_array(params, B), _pointers(u_in, B), _pointers(u_out, B),
+                                               _doubles(tau0, B), _doubles(dtau, B), int(nsteps), B,
                                                _stream(stream)))
 
 
@@ -223,12 +267,9 @@ def pino_physics_loss(g: Grid, params: Sequence, u_pred: Sequence, u_prev: Seque
     """PDE term of the PINO training loss (Sec. 3.5): loss[b] (a device float64 tensor of
     len(u_pred)) and, with grad, d loss[b] / d u_pred[b] into grad[b]."""
     B = len(u_pred)
-    P = (bs_params * B)(*[to_params(p) for p in params])
-    pp = (C.c_void_p * B)(*[_ptr(x) for x in u_pred])
-    pv = (C.c_void_p * B)(*[_ptr(x) for x in u_prev])
-    dt = (C.c_double * B)(*[float(t) for t in dtau])
-    pg = (C.c_void_p * B)(*[_ptr(x) for x in grad]) if grad is not None else None
-    return check(load().pino_physics_loss(g.h, P, pp, pv, dt, B, _ptr(loss), pg, _stream(stream)))
+    pg = _pointers(grad, B) if grad is not None else None
+    return check(load().pino_physics_loss(g.h, _params_array(params, B), _pointers(u_pred, B), _pointers(u_prev, B),
+                                          _doubles(dtau, B), B, _ptr(loss), pg, _stream(stream)))
 
 
 def bs_payoff3(M: int, xmax: float, p, u, stream=None):
@@ -242,11 +283,8 @@ def fine_propagate3(M: int, xmax: float, p, u_in: Sequence, u_out: Sequence, tau
     """F for three assets (19-point stencil) on len(u_in) states of M^3 nodes."""
     bp = to_params3(p)
     B = len(u_in)
-    pin = (C.c_void_p * B)(*[_ptr(x) for x in u_in])
-    pout = (C.c_void_p * B)(*[_ptr(x) for x in u_out])
-    t0 = (C.c_double * B)(*[float(t) for t in tau0])
-    return check(load().fine_propagate3(int(M), float(xmax), C.byref(bp), pin, pout, t0, B, float(dtau),
-                                        int(nsteps), _stream(stream)))
+    return check(load().fine_propagate3(int(M), float(xmax), C.byref(bp), _pointers(u_in, B), _pointers(u_out, B),
+                                        _doubles(tau0, B), B, float(dtau), int(nsteps), _stream(stream)))
 
 
 def coarse_propagate3(M: int, xmax: float, p, u_in, u_out, tau0: float, dtau_slice: float, nsteps: int,
@@ -310,12 +348,9 @@ def coarse_propagate_batched(g: Grid, kind: int, net, params: Sequence, u_in: Se
                              tau0: Sequence[float], dtau_slice: float, nsteps: int = 1, stream=None):
     """G on len(u_in) independent states at once (numerical: nsteps steps; PINO: the network)."""
     B = len(u_in)
-    bp = (bs_params * B)(*[to_params(p) for p in params])
-    ins = (C.c_void_p * B)(*[_ptr(u) for u in u_in])
-    outs = (C.c_void_p * B)(*[_ptr(u) for u in u_out])
-    t0 = (C.c_double * B)(*[float(t) for t in tau0])
-    return check(load().coarse_propagate_batched(g.h, int(kind), net.h if net is not None else None, bp, ins, outs,
-                                                 t0, float(dtau_slice), int(nsteps), B, _stream(stream)))
+    return check(load().coarse_propagate_batched(g.h, int(kind), net.h if net is not None else None,
+                                                 _params_array(params, B), _pointers(u_in, B), _pointers(u_out, B),
+                                                 _doubles(tau0, B), float(dtau_slice), int(nsteps), B, _stream(stream)))
 
 
 def parareal_sweep_range(g: Grid, p, N: int, coarse_steps: int, k: int, n_begin: int, n_end: int,

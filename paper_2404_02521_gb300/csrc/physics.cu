@@ -6,8 +6,8 @@
 //   r = (u~ - u_prev) / dtau - R_h u~ = ((u~ - u_prev) - dtau R_h u~) / dtau,
 //   loss = (1/n) sum r^2  (n = (M-1)^2),   d loss / d u~_i = (2/n) sum_j r_j d r_j / d u~_i.
 // Row j of R_h reads the 3 x 3 nodes around j, so the gradient at node i gathers the residuals
-// of the (up to) nine collocation points around i, each recomputed from u~; no scratch plane
-// is needed.  The residual is evaluated in FP32 from the same index-unit coefficients as the
+// of the (up to) nine collocation points around i from a tile in shared memory; no scratch
+// plane is needed.  The residual is evaluated in FP32 from the same index-unit coefficients as the
 // steppers (dtau R_h with the slice's dtau), the loss accumulated in FP64.
 #include "common.cuh"
 
@@ -26,6 +26,7 @@ struct PhysItem {
 
 constexpr int kPhysMaxItems = 32;
 constexpr int kPhysThreads = 256;
+constexpr size_t kPhysWideBlocks = 304;   // two blocks of the wide tile on every SM
 
 struct PhysBatch {
   PhysItem it[kPhysMaxItems];
@@ -33,87 +34,91 @@ struct PhysBatch {
   double inv_n;
 };
 
-// Coefficients of row (i, j) of dtau R_h: east, west, south (j + 1), north (j - 1), cross.
-struct RowW {
-  float e, w, s, n, g, rdt;
-};
-
-__device__ __forceinline__ RowW row_weights(const ItemDesc& d, int i, int j) {
-  RowW c;
-  float cgi, gj;
-  column_coefs(d, i, c.e, c.w, cgi);
-  row_coefs(d, j, c.s, c.n, gj);
-  c.g = cgi * gj;
-  c.rdt = d.rdt;
-  return c;
-}
-
-// r at collocation point (i, j).  Neighbours at x = 0 or y = 0 are read clamped: their
-// weights vanish there.
-__device__ __forceinline__ float residual_at(const PhysItem& it, int M, int i, int j) {
-  const float* u = it.pred;
-  const int il = i > 0 ? i - 1 : 0, ir = i + 1, jn = j > 0 ? j - 1 : 0, js = j + 1;
-  const RowW c = row_weights(it.d, i, j);
-  const float nW = u[jn * M + il], nC = u[jn * M + i], nE = u[jn * M + ir];
-  const float cW = u[j * M + il], cC = u[j * M + i], cE = u[j * M + ir];
-  const float sW = u[js * M + il], sC = u[js * M + i], sE = u[js * M + ir];
-  // dtau R_h u~ (eq. fd in index units)
-  const float t = c.e * (cE - cC) - c.w * (cC - cW) + c.s * (sC - cC) - c.n * (cC - nC) +
-                  c.g * ((sE - nE) - (sW - nW)) - c.rdt * cC;
-  return ((cC - it.prev[j * M + i]) - t) * it.rdtau;
-}
-
-// Weight with which row (i, j) of dtau R_h reads its neighbour at offset (di, dj).
-__device__ __forceinline__ float weight_at(const RowW& c, int di, int dj) {
-  if (di == 0 && dj == 0) return -(c.e + c.w + c.s + c.n + c.rdt);
-  if (dj == 0) return di > 0 ? c.e : c.w;
-  if (di == 0) return dj > 0 ? c.s : c.n;
-  return di == dj ? c.g : -c.g;   // (+1,+1), (-1,-1): +g; (+1,-1), (-1,+1): -g
-}
-
+// One block scores a tile of kPhysTile x kPhysTile nodes of one sample: the prediction is staged
+// with two nodes around the tile, the residuals are formed once on the tile and one node around
+// it, and the gradient gathers the nine around each node from shared memory.  Bound by the FP64
+// sum of r^2 and the latency of the three phases.  Recomputing the nine residuals at every node
+// from global memory, with an FP64 butterfly in every warp, took 21.1 us on the device for 32
+// samples of 128 x 128 (now 12.6) and 36 us for 4 of 512 x 512 (15.3).
+template <int kPhysTile>
 __global__ void __launch_bounds__(kPhysThreads) physics_loss_kernel(const __grid_constant__ PhysBatch pb) {
+  constexpr int kPhysP = kPhysTile + 4, kPhysR = kPhysTile + 2;
   const PhysItem& it = pb.it[blockIdx.y];
-  const int M = pb.M;
-  const int node = blockIdx.x * kPhysThreads + threadIdx.x;
+  const int M = pb.M, tid = threadIdx.x;
+  const int tiles = (M + kPhysTile - 1) / kPhysTile;
+  const int ty = blockIdx.x / tiles, i0 = (blockIdx.x - ty * tiles) * kPhysTile, j0 = ty * kPhysTile;
+  __shared__ float u[kPhysP * kPhysP], r[kPhysR * kPhysR];
+  for (int e = tid; e < kPhysP * kPhysP; e += kPhysThreads) {
+    const int row = e / kPhysP, c = e - row * kPhysP, i = i0 + c - 2, j = j0 + row - 2;
+    u[e] = i >= 0 && i < M && j >= 0 && j < M ? it.pred[j * M + i] : 0.f;
+  }
+  __syncthreads();
+  // r at the collocation points; a neighbour at index -1 has weight 0, its entry is the point's own
   double r2 = 0.0;
-  if (node < M * M) {
-    const int i = node % M, j = node / M;
-    const bool colloc = i <= M - 2 && j <= M - 2;
-    float own = 0.f;
-    if (colloc) {
-      own = residual_at(it, M, i, j);
-      r2 = (double)own * (double)own;
+  for (int e = tid; e < kPhysR * kPhysR; e += kPhysThreads) {
+    const int row = e / kPhysR, c = e - row * kPhysR, i = i0 + c - 1, j = j0 + row - 1;
+    float res = 0.f;
+    if (i >= 0 && j >= 0 && i <= M - 2 && j <= M - 2) {
+      float ce, cw, cgi, cs, cn, gj;
+      column_coefs(it.d, i, ce, cw, cgi);
+      row_coefs(it.d, j, cs, cn, gj);
+      const float* y = u + (row + 1) * kPhysP + c + 1;
+      const int w = i > 0 ? -1 : 0, n = j > 0 ? -kPhysP : 0;
+      const float nW = y[n + w], nC = y[n], nE = y[n + 1], cW = y[w], cC = y[0], cE = y[1];
+      const float sW = y[kPhysP + w], sC = y[kPhysP], sE = y[kPhysP + 1];
+      // dtau R_h u~ (eq. fd in index units)
+      const float t = ce * (cE - cC) - cw * (cC - cW) + cs * (sC - cC) - cn * (cC - nC) +
+                      (cgi * gj) * ((sE - nE) - (sW - nW)) - it.d.rdt * cC;
+      res = ((cC - it.prev[j * M + i]) - t) * it.rdtau;
+      if (c >= 1 && c <= kPhysTile && row >= 1 && row <= kPhysTile) r2 += (double)res * (double)res;
     }
-    if (it.grad) {
-      // d r_q / d u~_node = (delta - w_q(node - q)) / dtau over the collocation points q
-      // around the node
+    r[e] = res;
+  }
+  __syncthreads();
+  if (it.grad) {
+    // d r_q / d u~_node = (delta - w_q(node - q)) / dtau over the collocation points q around the
+    // node, w_q(o) the weight with which row q of dtau R_h reads its neighbour at offset o
+    for (int e = tid; e < kPhysTile * kPhysTile; e += kPhysThreads) {
+      const int row = e / kPhysTile, c = e % kPhysTile, i = i0 + c, j = j0 + row;
+      if (i >= M || j >= M) continue;
+      const float* y = r + (row + 1) * kPhysR + c + 1;
       float acc = 0.f;
+      float ce[3], cw[3], cg[3], cs[3], cn[3], gj[3];   // of the columns i-1..i+1 and rows j-1..j+1
+#pragma unroll
+      for (int o = 0; o < 3; ++o) {
+        column_coefs(it.d, i + o - 1, ce[o], cw[o], cg[o]);
+        row_coefs(it.d, j + o - 1, cs[o], cn[o], gj[o]);
+      }
+      // r is 0 at points outside the collocation set
 #pragma unroll
       for (int dj = -1; dj <= 1; ++dj) {
 #pragma unroll
         for (int di = -1; di <= 1; ++di) {
-          const int qi = i - di, qj = j - dj;   // the node is q's neighbour at (di, dj)
-          if (qi < 0 || qj < 0 || qi > M - 2 || qj > M - 2) continue;
-          const float rq = (di == 0 && dj == 0) ? own : residual_at(it, M, qi, qj);
-          const float w = weight_at(row_weights(it.d, qi, qj), di, dj);
+          const int qc = 1 - di, qr = 1 - dj;   // the node is q's neighbour at (di, dj)
+          const float rq = y[-dj * kPhysR - di];
+          float w;
+          if (di == 0 && dj == 0) w = -(ce[qc] + cw[qc] + cs[qr] + cn[qr] + it.d.rdt);
+          else if (dj == 0) w = di > 0 ? ce[qc] : cw[qc];
+          else if (di == 0) w = dj > 0 ? cs[qr] : cn[qr];
+          else w = di == dj ? cg[qc] * gj[qr] : -(cg[qc] * gj[qr]);
           acc = fmaf(rq, ((di == 0 && dj == 0) ? 1.f : 0.f) - w, acc);
         }
       }
-      it.grad[node] = (float)(2.0 * pb.inv_n) * acc * it.rdtau;
+      it.grad[j * M + i] = (float)(2.0 * pb.inv_n) * acc * it.rdtau;
     }
   }
-  // block sum of r^2 (FP64), one atomic per block
-  __shared__ double part[kPhysThreads / 32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) r2 += __shfl_down_sync(0xffffffffu, r2, o);
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = r2;
+  // block sum of r^2 (FP64), one atomic per block.  One warp folds the threads' sums from shared
+  // memory: a butterfly in every warp is three times the FP64 instructions.
+  __shared__ double part[kPhysThreads];
+  part[tid] = r2;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
+  if (tid >= 32) return;
+  double s = part[tid];
 #pragma unroll
-    for (int w = 0; w < kPhysThreads / 32; ++w) s += part[w];
-    if (s != 0.0) atomicAdd(it.loss, s * pb.inv_n);
-  }
+  for (int w = 1; w < kPhysThreads / 32; ++w) s += part[tid + 32 * w];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if (tid == 0 && s != 0.0) atomicAdd(it.loss, s * pb.inv_n);
 }
 
 }  // namespace
@@ -126,7 +131,6 @@ int launch_physics_loss(const bs_grid* g, const bs_params* p, const float* const
   pb.M = M;
   pb.inv_n = 1.0 / ((double)(M - 1) * (double)(M - 1));
   BS_CUDA_TRY(cudaMemsetAsync(loss, 0, sizeof(double) * (size_t)B, s));
-  const unsigned blocks = (unsigned)(((size_t)M * M + kPhysThreads - 1) / kPhysThreads);
   for (int base = 0; base < B; base += kPhysMaxItems) {
     const int nb = B - base < kPhysMaxItems ? B - base : kPhysMaxItems;
     for (int k = 0; k < nb; ++k) {
@@ -139,7 +143,14 @@ int launch_physics_loss(const bs_grid* g, const bs_params* p, const float* const
       it.d = make_item(p[b], 0.0, dtau[b]);
       it.rdtau = (float)(1.0 / dtau[b]);
     }
-    physics_loss_kernel<<<dim3(blocks, (unsigned)nb), kPhysThreads, 0, s>>>(pb);
+    // wide tiles recompute fewer residuals, narrow ones put more blocks on a chip that is not full
+    // (device time, 32 / 16 nodes: 32 of 128 x 128 12.6 / 14.7 us, 4 of 512 x 512 15.3 / 22.2;
+    // 8 of 128 x 128 8.8 / 8.5, 1 of 256 x 256 8.6 / 7.4, 4 of 64 x 64 8.4 / 6.4)
+    const unsigned t32 = (unsigned)(M + 31) / 32, t16 = (unsigned)(M + 15) / 16;
+    if ((size_t)t32 * t32 * nb >= kPhysWideBlocks)
+      physics_loss_kernel<32><<<dim3(t32 * t32, (unsigned)nb), kPhysThreads, 0, s>>>(pb);
+    else
+      physics_loss_kernel<16><<<dim3(t16 * t16, (unsigned)nb), kPhysThreads, 0, s>>>(pb);
     BS_CUDA_TRY(cudaGetLastError());
   }
   return BS_OK;
