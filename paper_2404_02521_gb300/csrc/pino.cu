@@ -7,7 +7,9 @@
 // mode with a complex C x C matrix; projection C -> H -> 1 with ReLU; the output is added to
 // u and the far-field data are set.  Batch normalisation is folded into W, b at load time.
 //
-// Every contraction runs on tcgen05 (umma.cuh), BF16 operands, FP32 accumulation:
+// States of up to 128 x 128 nodes run on a 128 x 128 network grid as one cluster per state
+// (pino_cluster.cu).  Larger ones run on 256 x 256 in the stages below.  Every contraction of the
+// stages runs on tcgen05 (umma.cuh), BF16 operands, FP32 accumulation:
 //   G1 x-DFT      [(c,y)]  x [x]          -> (kx, re/im)         N = 32 (24 used),  K = Mp
 //   G2 y-DFT      [(c,kx)] x [(y,re/im)]  -> (ky mode, re/im)    N = 64 (48 used),  K = 2 Mp
 //   G3 mixing     per mode: [state] x [(c,re/im)] -> (o,re/im)   N = 64, K = 64 (complex as
@@ -16,9 +18,6 @@
 //   G5 inv. x-DFT [pixel: x] x [(kx,re/im) of (o,y)] -> o, Hermitian weights and 1/Mp^2,
 //      + pointwise [pixel] x [c] -> o, both into one accumulator (K = 32 each); the
 //                 epilogue adds the bias and applies ReLU
-//      At Mp = 128 a tile is one row of pixels; before the last layer the same kernel then
-//      runs the next layer's G1 on the row (pino_pointwise_xdft_kernel), so only the first
-//      layer launches G1 on its own.
 //   P  projection [pixel]  x [c]          -> hidden, epilogue ReLU . w2 + b2, residual
 // Each epilogue writes the K-contiguous layout the next GEMM reads, so no transposes run
 // between them.  The DFT matrices are exact transforms (not learned) stored in BF16.
@@ -27,26 +26,15 @@
 #include <cstring>
 #include <vector>
 
-#include "common.cuh"
-#include "umma.cuh"
+#include "pino.cuh"
 
 namespace bsp {
-
-struct PinoState {
-  const float* in;     // state on its own grid (M x M)
-  float* out;          // PROP: output on the same grid
-  int M;
-  float h;             // grid spacing of in/out
-  float tau, dtau;     // network time inputs
-  float s1, s2, rho, r;
-  PayoffF pf;
-};
 
 enum { PAPPLY_PROP = 0, PAPPLY_INIT = 1, PAPPLY_ITER = 2, PAPPLY_ITER_SKIP = 3 };
 
 struct PinoRes {
   int Mp = 0, cap = 0, st_cap = 0;
-  bf16 *Ex = nullptr, *Ey = nullptr, *Eyi = nullptr, *Exi = nullptr;
+  bf16 *Ex = nullptr, *Ey = nullptr, *Eyi = nullptr, *Exi = nullptr;   // Mp = 128: canonical images, Ex with Exi
   bf16 *act_cp = nullptr, *act_pc = nullptr, *X1 = nullptr, *X2 = nullptr, *Y = nullptr, *Z1 = nullptr;
   float *wout = nullptr, *ump = nullptr;
   PinoState* st = nullptr;
@@ -64,6 +52,7 @@ struct bs_pino {
   bsp::bf16* W1;   // [H][C]
   float* b1;       // [H]
   float* w2;       // [H]
+  bsp::bf16 *mix, *Wpw_c, *W1_c;   // the cluster path's layouts of R, Wpw and W1 (pino.cuh); NULL for shapes it does not run
   float b2;
   int* err;
   bsp::PinoRes res[2];
@@ -86,6 +75,14 @@ static int upload(T** d, const std::vector<T>& h) {
 }
 
 static bf16 to_bf16(double x) { return __float2bfloat16((float)x); }
+
+// a rows x K matrix in the canonical K-major no-swizzle layout of its shared-memory tile
+static std::vector<bf16> canonical(const std::vector<bf16>& m, int rows, int K) {
+  std::vector<bf16> out((size_t)rows * K);
+  for (int r = 0; r < rows; ++r)
+    for (int k = 0; k < K; ++k) out[(size_t)canon_idx(r, k, K)] = m[(size_t)r * K + k];
+  return out;
+}
 
 // ---------------------------------------------------------------------------------------
 // Exact DFT matrices for a network grid Mp (host, FP64 -> BF16)
@@ -121,6 +118,17 @@ static int build_dft(bs_pino* net, PinoRes& R) {
       Eyi[(size_t)(2 * y + 1) * 48 + 2 * q + 1] = to_bf16(c);
     }
   int rc;
+  if (Mp == 128) {   // the cluster path's shared-memory images
+    const std::vector<bf16> xi = canonical(Exi, Mp, 32), x = canonical(Ex, 32, Mp);
+    Ex.assign(xi.begin(), xi.end());
+    Ex.insert(Ex.end(), x.begin(), x.end());
+    // the y-DFT's rows with the true 48 of 64, over (y, re/im)
+    Ey.resize((size_t)48 * 2 * Mp);
+    Ey = canonical(Ey, 48, 2 * Mp);
+    Eyi = canonical(Eyi, 2 * Mp, 48);
+    if ((rc = upload(&R.Ex, Ex)) || (rc = upload(&R.Ey, Ey)) || (rc = upload(&R.Eyi, Eyi))) return rc;
+    return BS_OK;
+  }
   if ((rc = upload(&R.Ex, Ex)) || (rc = upload(&R.Ey, Ey)) || (rc = upload(&R.Eyi, Eyi)) ||
       (rc = upload(&R.Exi, Exi)))
     return rc;
@@ -163,14 +171,16 @@ static int ensure_res(bs_pino* net, int Mp, int B, int nst, PinoRes** out) {
   if (!R.Ex && (rc = build_dft(net, R))) return rc;
   const size_t P = (size_t)Mp * Mp, C = net->C, mx = net->mx, MY = 2 * net->my;
   const size_t Bn = (size_t)B;
-  if ((rc = dev_alloc((void**)&R.act_cp, Bn * C * P * sizeof(bf16))) ||
-      (rc = dev_alloc((void**)&R.act_pc, Bn * C * P * sizeof(bf16))) ||
-      (rc = dev_alloc((void**)&R.X1, Bn * C * mx * 2 * Mp * sizeof(bf16))) ||
-      (rc = dev_alloc((void**)&R.X2, MY * mx * Bn * C * 2 * sizeof(bf16))) ||
-      (rc = dev_alloc((void**)&R.Y, Bn * C * mx * MY * 2 * sizeof(bf16))) ||
-      (rc = dev_alloc((void**)&R.Z1, Bn * C * Mp * mx * 2 * sizeof(bf16))) ||
-      (rc = dev_alloc((void**)&R.wout, Bn * P * sizeof(float))) ||
-      (rc = dev_alloc((void**)&R.ump, Bn * P * sizeof(float))) ||
+  if (Mp != 128 &&   // the cluster path keeps everything but the increment on the chip
+      ((rc = dev_alloc((void**)&R.act_cp, Bn * C * P * sizeof(bf16))) ||
+       (rc = dev_alloc((void**)&R.act_pc, Bn * C * P * sizeof(bf16))) ||
+       (rc = dev_alloc((void**)&R.X1, Bn * C * mx * 2 * Mp * sizeof(bf16))) ||
+       (rc = dev_alloc((void**)&R.X2, MY * mx * Bn * C * 2 * sizeof(bf16))) ||
+       (rc = dev_alloc((void**)&R.Y, Bn * C * mx * MY * 2 * sizeof(bf16))) ||
+       (rc = dev_alloc((void**)&R.Z1, Bn * C * Mp * mx * 2 * sizeof(bf16))) ||
+       (rc = dev_alloc((void**)&R.ump, Bn * P * sizeof(float)))))
+    return rc;
+  if ((rc = dev_alloc((void**)&R.wout, Bn * P * sizeof(float))) ||
       (rc = dev_alloc((void**)&R.st, (size_t)(nst > B ? nst : B) * sizeof(PinoState))))
     return rc;
   R.cap = B;
@@ -304,84 +314,6 @@ struct EpiAct {  // G5: rows pixels, cols o -> ReLU(spectral + W v + b) into bot
   }
 };
 
-// Mp = 128: the two-product stage of a layer and, in the same kernel, the next layer's x-DFT
-// of the tile's row (a tile is one row y of 128 pixels).  The tile's new activations go to
-// shared memory as the B operand [o][x] of a third product D3[(kx, re/im)][o] = Ex act^T
-// (accumulator columns 32..63), whose rows 0..23 are the x-DFT output of the row; the
-// channel-major copy of the activations, which only the x-DFT read, is not written.
-constexpr size_t kPwxSmem = 2 * ((size_t)2 * (128 + 32) * 32 + 128 * 128 + 32 * 128) + 64;
-
-__global__ void __launch_bounds__(128) pino_pointwise_xdft_kernel(PwOps<128> ops, const bf16* __restrict__ Ex,
-                                                                  const float* __restrict__ bias, bf16* act_pc,
-                                                                  bf16* X1, int* err) {
-  constexpr int Mp = 128, C = 32, P = Mp * Mp, mx = 12;
-  extern __shared__ __align__(1024) unsigned char smem[];
-  bf16* sA1 = reinterpret_cast<bf16*>(smem);
-  bf16* sB1 = sA1 + 128 * 32;
-  bf16* sA2 = sB1 + 32 * 32;
-  bf16* sB2 = sA2 + 128 * 32;
-  bf16* sA3 = sB2 + 32 * 32;    // x-DFT matrix rows (kx, re/im), K = x, zero below row 32
-  bf16* sB3 = sA3 + 128 * 128;  // the tile's activations [o][x]
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(sB3 + 32 * 128);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 1);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int b = blockIdx.y, y = blockIdx.x, x = tid;
-  ops.load(sA1, sB1, sA2, sB2);
-  for (int e = tid; e < 128 * 16; e += 128) {
-    const int r = e >> 4, kv = e & 15;
-    const bool ok = r < 32;
-    cp_async_16(sA3 + canon_idx(r, kv * 8, 128), ok ? Ex + (size_t)r * Mp + kv * 8 : Ex, ok);
-  }
-  asm volatile("cp.async.wait_all;\n" ::: "memory");
-  const uint32_t tmem = umma_setup<64>(tslot, mbar);
-  if (tid == 0) {
-    umma_issue<32>(tmem, smem_u32(sA1), smem_u32(sB1), 32, false);
-    umma_issue<32>(tmem, smem_u32(sA2), smem_u32(sB2), 32, true);
-    umma_commit(mbar);
-  }
-  const size_t p = (size_t)y * Mp + x;
-  if (umma_wait(mbar, err, 0)) {
-#pragma unroll 1
-    for (int c0 = 0; c0 < C; c0 += 16) {
-      float v[16];
-      umma_ld16(tmem, c0, v);
-      __align__(16) bf16 h[16];
-#pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        const int o = c0 + q;
-        h[q] = __float2bfloat16(fmaxf(v[q] + bias[o], 0.f));
-        sB3[canon_idx(o, x, 128)] = h[q];
-      }
-      uint4* dst = reinterpret_cast<uint4*>(act_pc + ((size_t)b * P + p) * C + c0);
-      dst[0] = reinterpret_cast<const uint4*>(h)[0];
-      dst[1] = reinterpret_cast<const uint4*>(h)[1];
-    }
-  }
-  // the activations, written by the threads, become the tensor cores' operand
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  if (tid == 0) {
-    umma_issue<32>(tmem + 32, smem_u32(sA3), smem_u32(sB3), 128, false);
-    umma_commit(mbar);
-  }
-  if (umma_wait(mbar, err, 1) && warp == 0) {
-#pragma unroll 1
-    for (int c0 = 0; c0 < C; c0 += 16) {
-      float v[16];
-      umma_ld16(tmem + 32, c0, v);   // lane = row (kx, re/im)
-      if (lane < 2 * mx) {
-        const int kx = lane >> 1, ri = lane & 1;
-#pragma unroll
-        for (int q = 0; q < 16; ++q)
-          X1[(((size_t)b * C + c0 + q) * mx + kx) * (2 * Mp) + 2 * y + ri] = __float2bfloat16(v[q]);
-      }
-    }
-  }
-  umma_teardown<64>(tmem);
-}
-
 struct ProjAcc { float s; };
 struct EpiProj { // P: rows pixels, cols hidden -> w = sum_h ReLU(v + b1) w2[h] + b2
   typedef ProjAcc Acc;
@@ -400,19 +332,6 @@ struct EpiProj { // P: rows pixels, cols hidden -> w = sum_h ReLU(v + b1) w2[h] 
 // ---------------------------------------------------------------------------------------
 // CUDA-core kernels: restriction, lifting, prolongation + residual + far field (+ Parareal)
 // ---------------------------------------------------------------------------------------
-
-// bilinear sample of a node field on an Mi grid at fractional node index (ti, tj)
-__device__ __forceinline__ float bilinear(const float* u, int Mi, float tx, float ty) {
-  int i0 = min((int)floorf(tx), Mi - 2), j0 = min((int)floorf(ty), Mi - 2);
-  i0 = max(i0, 0);
-  j0 = max(j0, 0);
-  const float fx = tx - i0, fy = ty - j0;
-  const float* r0 = u + (size_t)j0 * Mi;
-  const float* r1 = r0 + Mi;
-  const float a = r0[i0] * (1.f - fx) + r0[i0 + 1] * fx;
-  const float c = r1[i0] * (1.f - fx) + r1[i0 + 1] * fx;
-  return a * (1.f - fy) + c * fy;
-}
 
 __global__ void pino_restrict_kernel(const PinoState* st, float* ump, int Mp) {
   const int b = blockIdx.y;
@@ -545,19 +464,18 @@ __global__ void pino_defect_kernel(const double* partials, int nblocks, int pstr
 // ---------------------------------------------------------------------------------------
 #define BS_TRY_LAUNCH(expr) do { cudaError_t e_ = (expr); if (e_ != cudaSuccess) return cuda_error(e_, #expr); } while (0)
 
-template <int Mp>
-static int pino_network(bs_pino* net, PinoRes& R, const PinoState* st, int B, cudaStream_t s) {
-  constexpr int C = 32, mx = 12, MY = 24, P = Mp * Mp;
+// the staged path: a 256 x 256 network grid, whose activations (4 MB) a cluster cannot hold
+static int pino_network256(bs_pino* net, PinoRes& R, const PinoState* st, int B, cudaStream_t s) {
+  constexpr int Mp = 256, C = 32, mx = 12, MY = 24, P = Mp * Mp;
   const int pix_blocks = (P + 255) / 256;
   pino_lift_kernel<<<dim3(pix_blocks, B), 256, 0, s>>>(st, R.ump, net->lift_w, net->lift_b,
                                                        R.act_cp, R.act_pc, Mp, C, net->cin);
   BS_CUDA_TRY(cudaGetLastError());
   const int modes = MY * mx;
   for (int l = 0; l < net->L; ++l) {
-    // G1 (at Mp = 128 after the first layer it ran inside the previous layer's last stage)
-    if (Mp != 128 || l == 0)
-      BS_TRY_LAUNCH((launch_umma<32, Mp>(dim3(C * Mp / 128, B), GemmA{R.act_cp, (long long)C * P, Mp, C * Mp, Mp},
-                                         GemmB{R.Ex, 0, 0}, EpiX1{R.X1, Mp, mx, C}, net->err, s)));
+    // G1
+    BS_TRY_LAUNCH((launch_umma<32, Mp>(dim3(C * Mp / 128, B), GemmA{R.act_cp, (long long)C * P, Mp, C * Mp, Mp},
+                                       GemmB{R.Ex, 0, 0}, EpiX1{R.X1, Mp, mx, C}, net->err, s)));
     // G2
     BS_TRY_LAUNCH((launch_umma<64, 2 * Mp>(dim3((C * mx + 127) / 128, B),
                                            GemmA{R.X1, (long long)C * mx * 2 * Mp, 2 * Mp, C * mx, 2 * Mp},
@@ -570,23 +488,8 @@ static int pino_network(bs_pino* net, PinoRes& R, const PinoState* st, int B, cu
     BS_TRY_LAUNCH((launch_umma<kG4Chunk, 48>(dim3((C * mx + 127) / 128, B, (2 * Mp) / kG4Chunk),
                                              GemmA{R.Y, (long long)C * mx * MY * 2, MY * 2, C * mx, MY * 2},
                                              GemmB{R.Eyi, 0, kG4Chunk * 48}, EpiZ{R.Z1, Mp, mx, C}, net->err, s)));
-    // G5: inverse x-DFT and the pointwise product into one accumulator (at Mp = 128, before
-    // the last layer, with the next layer's x-DFT of the row)
+    // G5: inverse x-DFT and the pointwise product into one accumulator
     const PwOps<Mp> pw{R.Exi, R.Z1, R.act_pc, net->Wpw + (size_t)l * C * C};
-    if constexpr (Mp == 128) {
-      if (l + 1 < net->L) {
-        static bool attr_set = false;
-        if (!attr_set) {
-          BS_CUDA_TRY(cudaFuncSetAttribute(pino_pointwise_xdft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)kPwxSmem));
-          attr_set = true;
-        }
-        pino_pointwise_xdft_kernel<<<dim3(Mp, B), 128, kPwxSmem, s>>>(pw, R.Ex, net->pw_b + l * C, R.act_pc, R.X1,
-                                                                      net->err);
-        BS_CUDA_TRY(cudaGetLastError());
-        continue;
-      }
-    }
     BS_TRY_LAUNCH((launch_umma2<32, 32, 32>(dim3(P / 128, B), pw, EpiAct{R.act_cp, R.act_pc, net->pw_b + l * C, P, C},
                                             net->err, s)));
   }
@@ -616,10 +519,15 @@ static PinoState make_state(const ItemDesc& d, const float* in, float* out, int 
 static int pino_run(bs_pino* net, PinoRes& R, const PinoState* st, int B, int Mmax,
                     const ApplyArgs& aa, bool skip_net, cudaStream_t s) {
   const int Mp = R.Mp;
-  if (!skip_net) {
+  if (!skip_net && Mp == 128) {
+    const PinoClusterNet cn = {net->lift_w, net->lift_b, net->pw_b, net->b1, net->w2, R.Ex, R.Ey, R.Eyi,
+                               net->Wpw_c, net->W1_c, net->mix, net->b2, net->L, net->H};
+    const int rc = launch_pino_cluster(cn, st, R.wout, B, net->err, s);
+    if (rc) return rc;
+  } else if (!skip_net) {
     pino_restrict_kernel<<<dim3((Mp * Mp + 255) / 256, B), 256, 0, s>>>(st, R.ump, Mp);
     BS_CUDA_TRY(cudaGetLastError());
-    int rc = (Mp == 128) ? pino_network<128>(net, R, st, B, s) : pino_network<256>(net, R, st, B, s);
+    const int rc = pino_network256(net, R, st, B, s);
     if (rc) return rc;
   }
   pino_apply_kernel<<<dim3((Mmax * Mmax + 255) / 256, B), 256, 0, s>>>(st, R.wout, Mp, aa);
@@ -717,10 +625,10 @@ size_t pino_partials_bytes(int M, int N) {
   return (size_t)(N + 1) * nblocks * 2 * sizeof(double);
 }
 
-// kernels per network step on an M x M state: restrict, lift, 5 per layer (4 after the first
-// at Mp = 128), projection, apply
+// kernels per network step on an M x M state: the cluster kernel and apply, or restrict, lift,
+// 5 per layer, projection and apply
 int pino_launches_per_step(const bs_pino* net, int M) {
-  return network_grid(M) == 128 ? 5 + 4 * net->L : 4 + 5 * net->L;
+  return network_grid(M) == 128 ? 2 : 4 + 5 * net->L;
 }
 
 int pino_error_flag(const bs_pino* net, int* flag) {
@@ -787,6 +695,26 @@ extern "C" int pino_load(const char* path, bs_pino** out) {
   for (int c = 0; c < C; ++c)
     for (int h = 0; h < H; ++h) W1[(size_t)h * C + c] = __float2bfloat16(p1w[(size_t)c * H + h]);
   int rc;
+  if (C == 32 && mx == 12 && my == 12 && H % 16 == 0 && H <= 256) {
+    std::vector<bf16> mix((size_t)L * MYx * 2 * C * C), wc;
+    for (int l = 0; l < L; ++l) {
+      for (size_t m = 0; m < MYx; ++m)
+        for (int c = 0; c < C; ++c)
+          for (int o = 0; o < C; ++o) {
+            const size_t src = (((size_t)l * MYx + m) * C + c) * C + o;
+            mix[pino_mix_index(l, (int)m / mx, (int)m % mx, c, o, 0)] = __float2bfloat16(sre[src]);
+            mix[pino_mix_index(l, (int)m / mx, (int)m % mx, c, o, 1)] = __float2bfloat16(sim[src]);
+          }
+      const auto w = Wpw.begin() + (long)l * C * C;
+      const std::vector<bf16> one = canonical(std::vector<bf16>(w, w + C * C), C, C);
+      wc.insert(wc.end(), one.begin(), one.end());
+    }
+    if ((rc = upload(&net->mix, mix)) || (rc = upload(&net->Wpw_c, wc)) ||
+        (rc = upload(&net->W1_c, canonical(W1, H, C)))) {
+      pino_destroy(net);
+      return rc;
+    }
+  }
   if ((rc = upload(&net->lift_w, lift_w)) || (rc = upload(&net->lift_b, lift_b)) ||
       (rc = upload(&net->R, R)) || (rc = upload(&net->Wpw, Wpw)) || (rc = upload(&net->pw_b, pw_b)) ||
       (rc = upload(&net->W1, W1)) || (rc = upload(&net->b1, p1b)) || (rc = upload(&net->w2, p2w)) ||
@@ -801,7 +729,8 @@ extern "C" int pino_load(const char* path, bs_pino** out) {
 
 extern "C" int pino_destroy(bs_pino* net) {
   if (!net) return BS_OK;
-  void* ptrs[] = {net->lift_w, net->lift_b, net->R, net->Wpw, net->pw_b, net->W1, net->b1, net->w2, net->err};
+  void* ptrs[] = {net->lift_w, net->lift_b, net->R, net->Wpw, net->pw_b, net->W1, net->b1, net->w2, net->err,
+                  net->mix, net->Wpw_c, net->W1_c};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   free_res(net->res[0]);

@@ -48,7 +48,7 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint3
 }
 
 // element (r, k) of a rows x K tile in the canonical K-major no-swizzle layout
-__device__ __forceinline__ int canon_idx(int r, int k, int K) {
+__host__ __device__ __forceinline__ int canon_idx(int r, int k, int K) {
   return ((r >> 3) * (K >> 3) + (k >> 3)) * 64 + (r & 7) * 8 + (k & 7);
 }
 
@@ -118,13 +118,12 @@ __device__ __forceinline__ void umma_commit(uint64_t* mbar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(smem_u32(mbar)));
 }
 
-// Bounded wait for the products committed to mbar's phase of the given parity (0 for the
-// first commit, 1 for the second); records an error flag on time-out.
-__device__ __forceinline__ bool umma_wait(uint64_t* mbar, int* err, uint32_t parity = 0) {
+// Bounded wait for the products of mbar's first commit; records an error flag on time-out.
+__device__ __forceinline__ bool umma_wait(uint64_t* mbar, int* err) {
   uint32_t done = 0;
   for (int it = 0; it < kUmmaWaitIters && !done; ++it) {
     asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-                 : "=r"(done) : "r"(smem_u32(mbar)), "r"(parity) : "memory");
+                 : "=r"(done) : "r"(smem_u32(mbar)), "r"(0) : "memory");
   }
   if (!done && (threadIdx.x & 31) == 0) atomicExch(err, 1);
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
