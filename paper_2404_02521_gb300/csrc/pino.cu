@@ -52,6 +52,7 @@ struct bs_pino {
   bsp::bf16* W1;   // [H][C]
   float* b1;       // [H]
   float* w2;       // [H]
+  float b2_c;      // b2 + sum of b1 w2
   bsp::bf16 *mix, *Wpw_c, *W1_c;   // the cluster path's layouts of R, Wpw and W1 (pino.cuh); NULL for shapes it does not run
   float b2;
   int* err;
@@ -119,6 +120,8 @@ static int build_dft(bs_pino* net, PinoRes& R) {
     }
   int rc;
   if (Mp == 128) {   // the cluster path's shared-memory images
+    for (int x = 0; x < Mp; ++x)   // the columns that add the bias
+      for (int k = 24; k < 27; ++k) Exi[(size_t)x * 32 + k] = to_bf16(1.0);
     const std::vector<bf16> xi = canonical(Exi, Mp, 32), x = canonical(Ex, 32, Mp);
     Ex.assign(xi.begin(), xi.end());
     Ex.insert(Ex.end(), x.begin(), x.end());
@@ -521,7 +524,7 @@ static int pino_run(bs_pino* net, PinoRes& R, const PinoState* st, int B, int Mm
   const int Mp = R.Mp;
   if (!skip_net && Mp == 128) {
     const PinoClusterNet cn = {net->lift_w, net->lift_b, net->pw_b, net->b1, net->w2, R.Ex, R.Ey, R.Eyi,
-                               net->Wpw_c, net->W1_c, net->mix, net->b2, net->L, net->H};
+                               net->Wpw_c, net->W1_c, net->mix, net->b2_c, net->L, net->H};
     const int rc = launch_pino_cluster(cn, st, R.wout, B, net->err, s);
     if (rc) return rc;
   } else if (!skip_net) {
@@ -697,6 +700,9 @@ extern "C" int pino_load(const char* path, bs_pino** out) {
   int rc;
   if (C == 32 && mx == 12 && my == 12 && H % 16 == 0 && H <= 256) {
     std::vector<bf16> mix((size_t)L * MYx * 2 * C * C), wc;
+    double bw = p2b[0];
+    for (int h = 0; h < H; ++h) bw += (double)p1b[h] * p2w[h];
+    net->b2_c = (float)bw;
     for (int l = 0; l < L; ++l) {
       for (size_t m = 0; m < MYx; ++m)
         for (int c = 0; c < C; ++c)

@@ -33,22 +33,22 @@ __device__ __forceinline__ float bilinear(const float* u, int Mi, float tx, floa
 // Operands of the cluster path, laid out once as the shared-memory images it copies in.
 struct PinoClusterNet {
   const float *lift_w, *lift_b, *pw_b, *b1, *w2;
-  const bf16* dft_x;   // inverse x-DFT [128 x][32] then x-DFT [32][128 x], canonical
+  const bf16* dft_x;   // inverse x-DFT [128 x][32] (columns 24..26 one) then x-DFT [32][128 x], canonical
   const bf16* ey;      // y-DFT [48][256], canonical
   const bf16* eyi;     // inverse y-DFT [256][48], canonical
   const bf16* pw;      // [L][32][32] canonical (o, c)
   const bf16* w1;      // [H][32] canonical
   const bf16* mix;     // [L][72][2][4][4][32][4][2]: mode matrices, see pino_mix_index
-  float b2;
+  float b2;            // b2 + sum of b1 w2
   int L, H;
 };
 
 // Element (c -> o, re/im) of layer l's matrix of mode (q, kx) in PinoClusterNet::mix.  A unit is
-// four consecutive q at one kx; a warp's lane holds output o % 16 and half of the inputs.
+// four consecutive q at one kx; a lane holds four outputs and four inputs of a half unit.
 inline size_t pino_mix_index(int l, int q, int kx, int c, int o, int ri) {
-  const int unit = (q >> 2) * 12 + kx, lane = (c >> 4) * 16 + (o & 15);
-  return ((((((size_t)l * 72 + unit) * 2 + (o >> 4)) * 4 + (q & 3)) * 4 + ((c & 15) >> 2)) * 32 + lane) * 8 +
-         (size_t)(c & 3) * 2 + ri;
+  const int unit = (q >> 2) * 12 + kx, lane = (c >> 2) * 4 + ((o & 15) >> 2);
+  return ((((((size_t)l * 72 + unit) * 2 + (o >> 4)) * 4 + (q & 3)) * 4 + (c & 3)) * 32 + lane) * 8 +
+         (size_t)(o & 3) * 2 + ri;
 }
 
 // The network on B states (128 x 128 network grid): wout[b][y][x], the increment.

@@ -20,7 +20,9 @@
 // launches, activations through L2, 16k tiles of one MMA each per stage and scattered 2-byte
 // stores) and one state 170 us, nearly all of it launch and tile latency.  Here the tensor work
 // of a stage is a few dozen MMAs per CTA and the bound is the chain of stages: their epilogues and
-// three exchanges per layer: one state 55 us, 128 states 625 us (with the apply kernel).
+// three exchanges per layer: one state 48 us, 128 states 502 us (with the apply kernel).  Per layer at
+// CL = 8 (22 k cycles): MMAs 7.5 k (a 128 x N x 16 MMA takes 64 cycles and more at N = 32, the A tile's
+// fetch; the M-major ones 100), G3 3.6 k, exchanges 5 k, epilogues 4 k.
 //
 // An exchange needs no cluster barrier: the receiver's mbarrier counts the bytes, and a buffer
 // is rewritten only after a later exchange has proved that its readers are done (Y/Z/stage
@@ -48,21 +50,29 @@ struct PcCfg {
   // shared memory
   static constexpr int ACT = 0;                       // [G][x / 8][row][c / 8][x % 8][c % 8]
   static constexpr int YZ = ACT + G * 32768;          // stage of X1, then Y, then Z1
-  static constexpr int EA = YZ + 36864;               // x-DFTs, pointwise, inverse y-DFT | y-DFT | projection
-  static constexpr int EA_PW = EA + 16384, EA_EYI = EA + 18432;
+  static constexpr int EA = YZ + 36864;               // y-DFT | inverse x-DFT, pointwise, inverse y-DFT
+  static constexpr int EA_PW = EA + 8192, EA_EYI = EA + 10240;
+  // RECV holds X1 until G2 has read it, then mode matrices, in the last layer then the projection
   static constexpr int RECV = EA + 24576;             // X1 [source][(kx, c) / 8][y / 4][row % 8][16 B]
-  static constexpr int YST = RECV + ROWS * 1536;      // this CTA's part of Y
-  static constexpr int X2 = YST + HU * 256;           // [unit][q][c] (re, im)
-  static constexpr int FLT = X2 + NU * 512;           // lifting [4][32], bias [32], b1 [256], w2 [256]
-  static constexpr int BAR = FLT + 4 * (128 + 32 + 512);
-  static constexpr int SMEM = BAR + 192;
+  static constexpr int YST = RECV + (ROWS * 1536 > 16384 ? ROWS * 1536 : 16384);   // this CTA's part of Y
+  static constexpr int X2 = YST + HU * 256;           // [unit][q][c] (re, im); outside G2 .. G3 the x-DFT
+  static constexpr int FLT = X2 + 6144;               // lifting [4][32]
+  // mode matrices of G3 tasks that wait in shared memory: all of the next layer's if there is
+  // room, else 12 that follow the two per warp held in registers
+  static constexpr bool MIX_ALL = CL == 16;
+  static constexpr int MIX = MIX_ALL ? FLT + 512 : RECV;
+  static constexpr int MIX_TASKS = MIX_ALL ? 4 * HU : 12;
+  static_assert(NU * 512 <= 6144 && (MIX_ALL || MIX_TASKS * 2048 <= YST - RECV), "regions");
+  static constexpr int BAR = FLT + 512 + (MIX_ALL ? MIX_TASKS * 2048 : 0);
+  // (G1 reads 32 rows of the x-DFT and uses 24: the rest, too, lies within shared memory)
+  static constexpr int SMEM = BAR + 192 > X2 + 8192 ? BAR + 192 : X2 + 8192;
   static_assert(CL * XST <= 36864 && ROWS * 2048 <= 36864 && SMEM <= 232448, "shared memory");
   // G2 reads 128 rows of A and uses 12 CH of them: the rest lies within shared memory
   static_assert(RECV + (CL - 1) * XCH + (G / 2 - 1) * 256 + 16 * G * 128 <= SMEM, "rows beyond X1");
 };
 
 struct PcBars {
-  uint64_t g1[4], g5[4], pr[4], g2, g4, x1, x2, y, lda, ldy;
+  uint64_t g1[4], g5[4], pr[4], g2, g4, x1, x2, y, lda, ldy, ldx, ldm, ldw;
 };
 static_assert(sizeof(PcBars) <= 176, "barriers");
 
@@ -81,13 +91,32 @@ __device__ __forceinline__ void st_async_u32(uint32_t dst, uint32_t v, uint32_t 
                : "memory");
 }
 
-// one MMA of 128 x N x 16; a_mn: A is M-major
-__device__ __forceinline__ void pc_mma(uint32_t d, uint64_t a, uint64_t b, int N, bool a_mn, bool acc) {
-  const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn ? 1u : 0u) << 15) |
-                         ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-               " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-               ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc ? 1u : 0u));
+// A shared-memory operand descriptor in its two words; at(off) moves the start address.  Built
+// once per operand: a descriptor assembled from its fields before each MMA made the issuing
+// thread the bound (90 cycles per MMA; now an addition).
+struct PcDesc {
+  uint32_t lo, hi;
+  __device__ __forceinline__ PcDesc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
+    const uint64_t d = umma_desc(addr, lbo, sbo);
+    lo = (uint32_t)d;
+    hi = (uint32_t)(d >> 32);
+  }
+  __device__ __forceinline__ PcDesc at(uint32_t off) const {
+    PcDesc d = *this;
+    d.lo += off >> 4;
+    return d;
+  }
+};
+
+// one MMA of 128 x N x 16; A_MN: A is M-major
+constexpr uint32_t pc_idesc(int N, bool a_mn) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn ? 1u : 0u) << 15) | ((uint32_t)(N >> 3) << 17) |
+         ((uint32_t)(128 >> 4) << 24);
+}
+__device__ __forceinline__ void pc_mma(uint32_t d, const PcDesc& a, const PcDesc& b, uint32_t idesc, bool acc) {
+  asm volatile("{\n .reg .pred p;\n .reg .b64 da, db;\n setp.ne.b32 p, %6, 0;\n mov.b64 da, {%1, %2};\n"
+               " mov.b64 db, {%3, %4};\n tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}\n"
+               ::"r"(d), "r"(a.lo), "r"(a.hi), "r"(b.lo), "r"(b.hi), "r"(idesc), "r"(acc ? 1u : 0u));
 }
 
 // N consecutive accumulator columns of this warp's 32 lanes
@@ -113,9 +142,40 @@ __device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::befor
 __device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
 __device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 
+// a load of constant data that stays where it is written (ahead of a wait)
+__device__ __forceinline__ uint4 ld_early(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+
+// pairs of FP32 values, and the packed operations on them
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};\n" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;\n" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&v);
+}
+__device__ __forceinline__ uint32_t relu_bf16(uint32_t v) {   // (NaN gives 0)
+  const __nv_bfloat162 r = __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&v), __float2bfloat162_rn(0.f));
+  return *reinterpret_cast<const uint32_t*>(&r);
 }
 __device__ __forceinline__ float bf_lo(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
@@ -131,11 +191,9 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const PinoState*
   PcBars& bar = *reinterpret_cast<PcBars*>(smem + F::BAR);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(smem + F::BAR + 176);
   float* flift = reinterpret_cast<float*>(smem + F::FLT);
-  float* fbias = flift + 128;
-  float* fb1 = fbias + 32;
-  float* fw2 = fb1 + 256;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, set = warp >> 2, quad = warp & 3;
   const int rank = blockIdx.x, b = blockIdx.y, y0 = rank * ROWS;
+  const bool leader = quad == 0 && lane == 0;   // of the set
   const PinoState s = st[b];
   bool ok = true;
   auto wait1 = [&](uint64_t* mb, uint32_t parity) {   // one thread
@@ -149,6 +207,22 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const PinoState*
     __syncwarp();
   };
 
+  // this thread's nodes: column px of the rows r0 .. r0 + G - 1 of the group grp; their values of
+  // the state are in flight during the set-up.  The sets of a group need no others' progress
+  // between the inverse transform and the next x-DFT.
+  const int px = quad * 32 + lane, grp = set % G, r0 = set / G * G, yt = y0 + 4 * grp + r0;
+  float u[G];
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const int y = yt + g;
+    const float ratio = (float)(s.M - 1) / 127.f;
+    u[g] = s.M == 128 ? s.in[y * 128 + px] : bilinear(s.in, s.M, px * ratio, y * ratio);
+  }
+  const bf16* mix = net.mix + (size_t)(rank * F::HU * 4) * 1024;
+  auto load_mix_smem = [&](int l) {   // one thread
+    mbar_arm(&bar.ldm, F::MIX_TASKS * 2048);
+    bulk_g2s(sm + F::MIX, mix + ((size_t)l * 576 + (F::MIX_ALL ? 0 : 32)) * 1024, F::MIX_TASKS * 2048, &bar.ldm);
+  };
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;\n" ::"r"(smem_addr(tslot)));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
@@ -157,8 +231,11 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const PinoState*
     uint64_t* all = reinterpret_cast<uint64_t*>(&bar);
     for (int k = 0; k < (int)(sizeof(PcBars) / 8); ++k) mbar_init(all + k, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n");
-    mbar_arm(&bar.lda, 16384);
-    bulk_g2s(sm + F::EA, net.dft_x, 16384, &bar.lda);
+    mbar_arm(&bar.ldx, 6144);
+    bulk_g2s(sm + F::X2, net.dft_x + 4096, 6144, &bar.ldx);
+    mbar_arm(&bar.ldy, 24576);
+    bulk_g2s(sm + F::EA, net.ey, 24576, &bar.ldy);
+    if (F::MIX_ALL) load_mix_smem(0);
     mbar_arm(&bar.x1, ROWS * 1536);
     mbar_arm(&bar.x2, F::NU * 512);
     mbar_arm(&bar.y, 36864);
@@ -174,10 +251,6 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const PinoState*
 #pragma unroll
     for (int c = 0; c < 3; ++c) flift[32 * (c + 1) + o] = net.lift_w[c * 32 + o];
   }
-  for (int k = tid; k < net.H; k += kPcThreads) {
-    fb1[k] = net.b1[k];
-    fw2[k] = net.w2[k];
-  }
   tc_before();
   __syncthreads();
   tc_after();
@@ -185,18 +258,10 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const PinoState*
   const uint32_t tlane = tmem + ((uint32_t)(quad * 32) << 16);
   cluster_arrive();   // the barriers of every CTA exist before the first exchange
 
-  // this thread's node column, and where its 16 bytes of channels 8 cc .. of row 4 g + set lie
-  const int px = quad * 32 + lane;
-  unsigned char* act_px = smem + F::ACT + (px >> 3) * 2048 + set * 512 + (px & 7) * 16;
+  // where 16 bytes of channels 8 cc .. of this thread's nodes lie
+  unsigned char* act_px = smem + F::ACT + grp * 32768 + (px >> 3) * 2048 + r0 * 512 + (px & 7) * 16;
   {
     const float hp = s.h * (float)(s.M - 1) / 127.f;   // network grid spacing
-    const float ratio = (float)(s.M - 1) / 127.f;
-    float u[G];
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      const int y = y0 + 4 * g + set;
-      u[g] = s.M == 128 ? s.in[y * 128 + px] : bilinear(s.in, s.M, px * ratio, y * ratio);
-    }
 #pragma unroll
     for (int cc = 0; cc < 4; ++cc) {
       float base[8], wu[8], wy[8];
@@ -209,33 +274,33 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const PinoState*
       }
 #pragma unroll
       for (int g = 0; g < G; ++g) {
-        const float y = (float)(y0 + 4 * g + set) * hp;
+        const float y = (float)(yt + g) * hp;
         uint32_t h[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k)
           h[k] = pack_bf16(fmaf(u[g], wu[2 * k], fmaf(y, wy[2 * k], base[2 * k])),
                            fmaf(u[g], wu[2 * k + 1], fmaf(y, wy[2 * k + 1], base[2 * k + 1])));
-        *reinterpret_cast<uint4*>(act_px + g * 32768 + cc * 128) = make_uint4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<uint4*>(act_px + g * 512 + cc * 128) = make_uint4(h[0], h[1], h[2], h[3]);
       }
     }
   }
 
   // G1 of group g: D[(row, c)][(kx, re/im)] in the columns of the group's first row
   auto issue_g1 = [&](int g) {
-#pragma unroll 1
+    const PcDesc a(sm + F::ACT + g * 32768, 2048, 128), x(sm + F::X2, 128, 2048);
+#pragma unroll
     for (int kk = 0; kk < 8; ++kk)
-      pc_mma(tmem + g * 128, umma_desc(sm + F::ACT + g * 32768 + kk * 4096, 2048, 128),
-             umma_desc(sm + F::EA + 8192 + kk * 256, 128, 2048), 32, true, kk > 0);
+      pc_mma(tmem + g * 128, a.at(kk * 4096), x.at(kk * 256), pc_idesc(32, true), kk > 0);
     umma_commit(&bar.g1[g]);
   };
   proxy_fence();
   tc_before();
   __syncthreads();
   cluster_wait();
-  if (tid == 0) {
+  if (leader && set < G) {
     tc_after();
-    wait1(&bar.lda, 0);
-    for (int g = 0; g < G; ++g) issue_g1(g);
+    wait1(&bar.ldx, 0);
+    issue_g1(set);
   }
   __syncwarp();
 
@@ -247,6 +312,10 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const PinoState*
       constexpr int HV = G == 4 ? 2 : 1;   // halves of kx per thread
       const int g = set % G;
       wait(&bar.g1[g], par);
+      if (l > 0) {   // the stage takes the place of Z1
+#pragma unroll
+        for (int k = 0; k < G; ++k) wait(&bar.g5[k], par ^ 1);
+      }
       tc_after();
       const int dst = lane / F::CH, cl = lane % F::CH;
       uint32_t v[HV][16];
@@ -268,52 +337,48 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const PinoState*
         }
       }
     }
-    if (tid < 32) fbias[tid] = net.pw_b[l * 32 + tid];
     proxy_fence();
     tc_before();
     __syncthreads();
+    if (warp < CL && lane == 0)   // a copy per warp: one warp issuing them all took 1000 cycles
+      bulk_s2c(cluster_addr(sm + F::RECV + rank * F::XCH, warp), sm + F::YZ + warp * F::XST, F::XCH,
+               cluster_addr(smem_addr(&bar.x1), warp));
+    __syncwarp();
     if (warp == 0) {
-      // every G1 is complete: the x-DFT's region takes the y-DFT
-      if (lane == 0) {
-        mbar_arm(&bar.ldy, 24576);
-        bulk_g2s(sm + F::EA, net.ey, 24576, &bar.ldy);
-      }
-      if (lane < CL)
-        bulk_s2c(cluster_addr(sm + F::RECV + rank * F::XCH, lane), sm + F::YZ + lane * F::XST, F::XCH,
-                 cluster_addr(smem_addr(&bar.x1), lane));
       // ---- G2
       if (lane == 0) {
         wait1(&bar.ldy, par);
         wait1(&bar.x1, par);
         mbar_arm(&bar.x1, ROWS * 1536);
         tc_after();
-#pragma unroll 1
-        for (int k = 0; k < 16; ++k) {
-          const int src = k / (G / 2), ks = k % (G / 2);
-          pc_mma(tmem, umma_desc(sm + F::RECV + src * F::XCH + ks * 256, 128, G * 128),
-                 umma_desc(sm + F::EA + k * 256, 128, 4096), 48, false, k > 0);
-        }
+        const PcDesc a(sm + F::RECV, 128, G * 128), e(sm + F::EA, 128, 4096);
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          pc_mma(tmem, a.at(k / (G / 2) * F::XCH + k % (G / 2) * 256), e.at(k * 256), pc_idesc(48, false), k > 0);
         umma_commit(&bar.g2);
       }
       __syncwarp();
     }
     // the first mode matrices of G3, in flight meanwhile
-    const bf16* mix = net.mix + (size_t)l * (72 * 2 * 4 * 1024) + lane * 8;
-    uint4 wv[4];
-    auto load_mix = [&](int task) {
-      const uint4* p = reinterpret_cast<const uint4*>(mix + ((size_t)(rank * F::HU + (task >> 2)) * 4 + (task & 3)) * 1024);
+    uint4 wa[4], wb[4];
+    auto load_mix = [&](uint4 (&wv)[4], int task) {
+      const uint4* p = reinterpret_cast<const uint4*>(mix + ((size_t)l * 576 + task) * 1024 + lane * 8);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) wv[j] = __ldg(p + 32 * j);
+      for (int j = 0; j < 4; ++j) wv[j] = ld_early(p + 32 * j);
     };
-    load_mix(warp);
+    if (!F::MIX_ALL) {
+      load_mix(wa, warp);
+      load_mix(wb, warp + 16);
+    }
     // ---- X2: lane = (kx, c), columns (q, re/im); a value goes to the CTA(s) that mix its mode
     wait(&bar.g2, par);
     tc_after();
     if (tid == 0) {
-      // G2 has read the y-DFT: its region takes back the x-DFTs, and the layer's other operands
+      // G2 has read the y-DFT and X1: their regions take the operands of the stages that follow
       constexpr uint32_t kEyi = ROWS * 2 * 96;
-      mbar_arm(&bar.lda, 16384 + 2048 + kEyi);
-      bulk_g2s(sm + F::EA, net.dft_x, 16384, &bar.lda);
+      if (!F::MIX_ALL) load_mix_smem(l);
+      mbar_arm(&bar.lda, 8192 + 2048 + kEyi);
+      bulk_g2s(sm + F::EA, net.dft_x, 8192, &bar.lda);
       bulk_g2s(sm + F::EA_PW, net.pw + (size_t)l * 1024, 2048, &bar.lda);
       bulk_g2s(sm + F::EA_EYI, net.eyi + (size_t)rank * (kEyi / 2), kEyi, &bar.lda);
     }
@@ -339,55 +404,115 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const PinoState*
         }
       }
     }
-    // ---- G3: a warp per (half unit, q); lane = output o % 16 and half of the inputs
+    // ---- G3: a warp per (half unit, q); a lane multiplies 4 inputs into 4 outputs, so that its inputs
+    // are one shared-memory read (a broadcast read per input and output pair made the return path to
+    // the registers the bound: 4800 cycles at CL = 8)
     wait(&bar.x2, par);
     if (tid == 0) mbar_arm(&bar.x2, F::NU * 512);
     __syncwarp();
-#pragma unroll 1
-    for (int task = warp; task < 4 * F::HU; task += kPcThreads / 32) {
+    auto mix_task = [&](uint4 (&wv)[4], int task, int next) {
       const int hu = task >> 2, q = task & 3, unit = (rank * F::HU + hu) >> 1, u0 = rank * F::HU / 2;
-      uint4 w[4];
+      const uint4 xv = *reinterpret_cast<const uint4*>(smem + F::X2 + ((unit - u0) * 4 + q) * 128 + (lane >> 2) * 16);
+      const uint32_t xs[4] = {xv.x, xv.y, xv.z, xv.w};
+      uint64_t br[4] = {0, 0, 0, 0}, bi[4] = {0, 0, 0, 0};   // the sums of re(x) (wr, wi) and of im(x) (wr, wi)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) w[j] = wv[j];
-      if (task + kPcThreads / 32 < 4 * F::HU) load_mix(task + kPcThreads / 32);
-      const uint4* xp = reinterpret_cast<const uint4*>(smem + F::X2 + ((unit - u0) * 4 + q) * 128 + (lane >> 4) * 64);
-      float re = 0.f, im = 0.f;
+      for (int i = 0; i < 4; ++i) {
+        const uint64_t xr = pack2(bf_lo(xs[i]), bf_lo(xs[i])), xi = pack2(bf_hi(xs[i]), bf_hi(xs[i]));
+        const uint32_t ws[4] = {wv[i].x, wv[i].y, wv[i].z, wv[i].w};
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const uint4 xv = xp[j];
-        const uint32_t xs[4] = {xv.x, xv.y, xv.z, xv.w}, ws[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float xr = bf_lo(xs[i]), xi = bf_hi(xs[i]), wr = bf_lo(ws[i]), wi = bf_hi(ws[i]);
-          re = fmaf(-xi, wi, fmaf(xr, wr, re));
-          im = fmaf(xi, wr, fmaf(xr, wi, im));
+        for (int o = 0; o < 4; ++o) {
+          const uint64_t w = pack2(bf_lo(ws[o]), bf_hi(ws[o]));
+          br[o] = fma2(xr, w, br[o]);
+          bi[o] = fma2(xi, w, bi[o]);
         }
       }
-      re += __shfl_xor_sync(0xffffffffu, re, 16);
-      im += __shfl_xor_sync(0xffffffffu, im, 16);
-      if (lane < 16)
-        *reinterpret_cast<uint32_t*>(smem + F::YST + hu * 256 + (lane >> 3) * 128 + (lane & 7) * 16 + q * 4) =
-            pack_bf16(re, im);
+      if (next < 4 * F::HU) load_mix(wv, next);
+      float re[4], im[4];
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        float rr, ri, ir, ii;
+        unpack2(br[o], rr, ri);
+        unpack2(bi[o], ir, ii);
+        re[o] = rr - ii;
+        im[o] = ri + ir;
+      }
+      // sum over the eight lanes of the same outputs, halving what a lane holds: lane bits 4 and 3
+      // choose the output, bit 2 re or im
+      const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+#pragma unroll
+      for (int o = 0; o < 2; ++o) {
+        const float sr = __shfl_xor_sync(0xffffffffu, h4 ? re[o] : re[o + 2], 16);
+        const float si = __shfl_xor_sync(0xffffffffu, h4 ? im[o] : im[o + 2], 16);
+        re[o] = (h4 ? re[o + 2] : re[o]) + sr;
+        im[o] = (h4 ? im[o + 2] : im[o]) + si;
+      }
+      const float sr = __shfl_xor_sync(0xffffffffu, h3 ? re[0] : re[1], 8);
+      const float si = __shfl_xor_sync(0xffffffffu, h3 ? im[0] : im[1], 8);
+      const float r1 = (h3 ? re[1] : re[0]) + sr, i1 = (h3 ? im[1] : im[0]) + si;
+      const float v = (h2 ? i1 : r1) + __shfl_xor_sync(0xffffffffu, h2 ? r1 : i1, 4);
+      const float vi = __shfl_xor_sync(0xffffffffu, v, 4);
+      const int o = (lane & 3) * 4 + (h4 ? 2 : 0) + (h3 ? 1 : 0);
+      if (!h2)
+        *reinterpret_cast<uint32_t*>(smem + F::YST + hu * 256 + (o >> 3) * 128 + (o & 7) * 16 + q * 4) = pack_bf16(v, vi);
+    };
+    auto smem_mix = [&](uint4 (&wv)[4], int k) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        wv[j] = *reinterpret_cast<const uint4*>(smem + F::MIX + k * 2048 + j * 512 + lane * 16);
+    };
+    constexpr int kNone = 1 << 20;
+    if (F::MIX_ALL) {
+      wait(&bar.ldm, par);
+#pragma unroll 1
+      for (int task = warp; task < F::MIX_TASKS; task += 16) {
+        smem_mix(wa, task);
+        mix_task(wa, task, kNone);
+      }
+    } else {
+      constexpr int kRest = 32 + F::MIX_TASKS;   // the tasks after those in registers and shared memory
+      mix_task(wa, warp, kRest + warp);
+      mix_task(wb, warp + 16, kRest + 16 + warp);
+      if (warp < F::MIX_TASKS) {
+        uint4 wc[4];
+        wait(&bar.ldm, par);
+        smem_mix(wc, warp);
+        mix_task(wc, 32 + warp, kNone);
+      }
+      mix_task(wa, kRest + warp, kNone);
+      if (kRest + 16 + warp < 4 * F::HU) mix_task(wb, kRest + 16 + warp, kNone);
+      static_assert(F::MIX_ALL || (kRest + 16 <= 4 * F::HU && 4 * F::HU <= kRest + 32), "tasks");
     }
     proxy_fence();
     tc_before();
     __syncthreads();
+    if (warp < CL && lane == 0)
+      bulk_s2c(cluster_addr(sm + F::YZ + rank * (F::HU * 256), warp), sm + F::YST, F::HU * 256,
+               cluster_addr(smem_addr(&bar.y), warp));
+    __syncwarp();
+    if (tid == 0) {   // G3 has read X2 and the mode matrices
+      if (l + 1 < net.L) {
+        mbar_arm(&bar.ldx, 6144);
+        bulk_g2s(sm + F::X2, net.dft_x + 4096, 6144, &bar.ldx);
+        if (F::MIX_ALL) load_mix_smem(l + 1);
+      } else {
+        mbar_arm(&bar.ldw, net.H * 64);
+        bulk_g2s(sm + F::RECV, net.w1, net.H * 64, &bar.ldw);
+      }
+    }
+    __syncwarp();
     if (warp == 0) {
-      if (lane < CL)
-        bulk_s2c(cluster_addr(sm + F::YZ + rank * (F::HU * 256), lane), sm + F::YST, F::HU * 256,
-                 cluster_addr(smem_addr(&bar.y), lane));
       // ---- G4
       if (lane == 0) {
-        wait1(&bar.lda, (l + 1) & 1);
+        wait1(&bar.lda, par);
         wait1(&bar.y, par);
         mbar_arm(&bar.y, 36864);
         tc_after();
-#pragma unroll 1
+        const PcDesc a(sm + F::YZ, 6144, 128), e(sm + F::EA_EYI, 128, 768);
+#pragma unroll
         for (int t = 0; t < 3; ++t)
-#pragma unroll 1
+#pragma unroll
           for (int kk = 0; kk < 3; ++kk)
-            pc_mma(tmem + 64 + t * 32, umma_desc(sm + F::YZ + t * 2048 + kk * 12288, 6144, 128),
-                   umma_desc(sm + F::EA_EYI + kk * 256, 128, 768), 2 * ROWS, false, kk > 0);
+            pc_mma(tmem + 64 + t * 32, a.at(t * 2048 + kk * 12288), e.at(kk * 256), pc_idesc(2 * ROWS, false), kk > 0);
         umma_commit(&bar.g4);
       }
       __syncwarp();
@@ -407,42 +532,43 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const PinoState*
         for (int i = 0; i < G; ++i)
           *reinterpret_cast<uint32_t*>(z + (set * G + i) * 2048 + t * 128) =
               pack_bf16(__uint_as_float(v[t][2 * i]), __uint_as_float(v[t][2 * i + 1]));
-      // K = 24 .. 31 is padding
-      if (tid < ROWS * 32)
+      // K = 24 .. 31: the bias in three parts, exactly, against ones in the inverse x-DFT
+      if (tid < ROWS * 32) {
+        const float bias = net.pw_b[l * 32 + lane];
+        const float hi = bf_lo(pack_bf16(bias, 0.f));
+        const bool fin = fabsf(hi) < INFINITY;
+        const float mid = fin ? bf_lo(pack_bf16(bias - hi, 0.f)) : 0.f, lo = fin ? (bias - hi) - mid : 0.f;
         *reinterpret_cast<uint4*>(smem + F::YZ + (tid >> 5) * 2048 + (lane >> 3) * 512 + 384 + (lane & 7) * 16) =
-            make_uint4(0, 0, 0, 0);
+            make_uint4(pack_bf16(hi, mid), pack_bf16(lo, 0.f), 0, 0);
+      }
     }
     proxy_fence();
     tc_before();
     __syncthreads();
-    // ---- G5
-    if (tid == 0) {
+    // ---- G5: the leader of a set issues its group.  The inverse x-DFT of the group's four rows
+    // is one product (N = 4 rows x 32 outputs), the pointwise products follow row by row
+    if (leader && set < G) {
       tc_after();
-#pragma unroll 1
-      for (int g = 0; g < G; ++g) {
-#pragma unroll 1
-        for (int r = 0; r < 4; ++r) {
-          const uint32_t d = tmem + (g * 4 + r) * 32;
+      const uint32_t d = tmem + set * 128;
+      const PcDesc x(sm + F::EA, 128, 512), z(sm + F::YZ + set * 8192, 128, 512);
+      const PcDesc a(sm + F::ACT + set * 32768, 128, 2048), w(sm + F::EA_PW, 128, 512);
 #pragma unroll
-          for (int kk = 0; kk < 2; ++kk)
-            pc_mma(d, umma_desc(sm + F::EA + kk * 256, 128, 512),
-                   umma_desc(sm + F::YZ + (g * 4 + r) * 2048 + kk * 256, 128, 512), 32, false, kk > 0);
+      for (int kk = 0; kk < 2; ++kk) pc_mma(d, x.at(kk * 256), z.at(kk * 256), pc_idesc(128, false), kk > 0);
 #pragma unroll
-          for (int kk = 0; kk < 2; ++kk)
-            pc_mma(d, umma_desc(sm + F::ACT + g * 32768 + r * 512 + kk * 256, 128, 2048),
-                   umma_desc(sm + F::EA_PW + kk * 256, 128, 512), 32, false, true);
-        }
-        umma_commit(&bar.g5[g]);
-      }
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk)
+          pc_mma(d + r * 32, a.at(r * 512 + kk * 256), w.at(kk * 256), pc_idesc(32, false), true);
+      umma_commit(&bar.g5[set]);
     }
     __syncwarp();
+    wait(&bar.g5[grp], par);
+    tc_after();
 #pragma unroll 1
     for (int g = 0; g < G; ++g) {
-      wait(&bar.g5[g], par);
-      tc_after();
       uint32_t v[2][16];
-      pc_ld<16>(tlane + (g * 4 + set) * 32, v[0]);
-      pc_ld<16>(tlane + (g * 4 + set) * 32 + 16, v[1]);
+      pc_ld<16>(tlane + (grp * 4 + r0 + g) * 32, v[0]);
+      pc_ld<16>(tlane + (grp * 4 + r0 + g) * 32 + 16, v[1]);
       pc_ld_wait();
 #pragma unroll
       for (int cc = 0; cc < 4; ++cc) {
@@ -450,63 +576,87 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const PinoState*
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const int o = cc * 8 + 2 * k;
-          h[k] = pack_bf16(fmaxf(__uint_as_float(v[o >> 4][o & 15]) + fbias[o], 0.f),
-                           fmaxf(__uint_as_float(v[o >> 4][(o & 15) + 1]) + fbias[o + 1], 0.f));
+          h[k] = relu_bf16(pack_bf16(__uint_as_float(v[o >> 4][o & 15]), __uint_as_float(v[o >> 4][(o & 15) + 1])));
         }
-        *reinterpret_cast<uint4*>(act_px + g * 32768 + cc * 128) = make_uint4(h[0], h[1], h[2], h[3]);
-      }
-      proxy_fence();
-      tc_before();
-      __syncthreads();
-      if (l + 1 < net.L) {
-        if (tid == 0) {
-          tc_after();
-          issue_g1(g);
-        }
-        __syncwarp();
+        *reinterpret_cast<uint4*>(act_px + g * 512 + cc * 128) = make_uint4(h[0], h[1], h[2], h[3]);
       }
     }
-  }
-
-  // ---- projection: set takes a row of each group, its first thread issues the row's products
-  if (tid == 0) {
-    mbar_arm(&bar.lda, net.H * 64);
-    bulk_g2s(sm + F::EA, net.w1, net.H * 64, &bar.lda);
-  }
-  __syncwarp();
-  wait(&bar.lda, (net.L + 1) & 1);
-  uint32_t ppar = 0;
-#pragma unroll 1
-  for (int g = 0; g < G; ++g) {
-    float acc = 0.f;
-#pragma unroll 1
-    for (int h0 = 0; h0 < net.H; h0 += 128) {
-      const int n = min(128, net.H - h0);
-      if (quad == 0 && lane == 0) {
+    proxy_fence();
+    tc_before();
+    if (l + 1 < net.L) {
+      asm volatile("bar.sync %0, %1;\n" ::"r"(1 + grp), "n"(512 / G) : "memory");   // the group's sets
+      if (leader && set < G) {
         tc_after();
+        wait1(&bar.ldx, par ^ 1);
+        issue_g1(set);
+      }
+      if (tid == 0) {   // the inverse x-DFT and pointwise operands make way for the y-DFT
+        for (int k = 0; k < G; ++k) wait1(&bar.g5[k], par);
+        mbar_arm(&bar.ldy, 24576);
+        bulk_g2s(sm + F::EA, net.ey, 24576, &bar.ldy);
+      }
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+
+  // ---- projection, 128 hidden nodes at a time for the four rows of a group: each set takes 32 hidden
+  // nodes, whose biases and weights it keeps in registers, and the sets' sums meet in shared
+  // memory (with a set per row every bias and weight is a shared-memory or constant-bank read per
+  // row: 4200 and 4600 cycles per group, now 3600).  ReLU(v + b) w = max(v, -b) w + b w, the sum of b w in net.b2.
+  wait(&bar.ldw, 0);
+  float* part = reinterpret_cast<float*>(smem + F::YZ);   // [set][row][128]
+  uint32_t ppar = 0;
+  const PcDesc pa(sm + F::ACT, 128, 2048), pw(sm + F::RECV, 128, 512);
+#pragma unroll 1
+  for (int h0 = 0; h0 < net.H; h0 += 128) {
+    const int n = min(128, net.H - h0);
+    float nb[32], w2[32];
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+      const int h = set * 32 + k;
+      nb[k] = h < n ? -net.b1[h0 + h] : 0.f;
+      w2[k] = h < n ? net.w2[h0 + h] : 0.f;
+    }
+#pragma unroll 1
+    for (int g = 0; g < G; ++g) {
+      if (leader) {   // of set: row set of the group
+        tc_after();
+        const uint32_t idesc = pc_idesc(0, false) | ((uint32_t)(n >> 3) << 17);
 #pragma unroll
         for (int kk = 0; kk < 2; ++kk)
-          pc_mma(tmem + set * 128, umma_desc(sm + F::ACT + g * 32768 + set * 512 + kk * 256, 128, 2048),
-                 umma_desc(sm + F::EA + h0 * 64 + kk * 256, 128, 512), n, false, kk > 0);
+          pc_mma(tmem + set * 128, pa.at(g * 32768 + set * 512 + kk * 256), pw.at(h0 * 64 + kk * 256), idesc, kk > 0);
         umma_commit(&bar.pr[set]);
       }
       __syncwarp();
-      wait(&bar.pr[set], ppar);
-      ppar ^= 1;
-      tc_after();
 #pragma unroll 1
-      for (int c0 = 0; c0 < n; c0 += 16) {
-        uint32_t v[16];
-        pc_ld<16>(tlane + set * 128 + c0, v);
-        pc_ld_wait();
+      for (int r = 0; r < 4; ++r) {
+        wait(&bar.pr[r], ppar);
+        tc_after();
+        float acc = 0.f, acc1 = 0.f;
 #pragma unroll
-        for (int k = 0; k < 16; ++k)
-          acc = fmaf(fmaxf(__uint_as_float(v[k]) + fb1[h0 + c0 + k], 0.f), fw2[h0 + c0 + k], acc);
+        for (int c0 = 0; c0 < 32; c0 += 16) {
+          if (set * 32 + c0 >= n) break;
+          uint32_t v[16];
+          pc_ld<16>(tlane + r * 128 + set * 32 + c0, v);
+          pc_ld_wait();
+#pragma unroll
+          for (int k = 0; k < 16; k += 2) {
+            acc = fmaf(fmaxf(__uint_as_float(v[k]), nb[c0 + k]), w2[c0 + k], acc);
+            acc1 = fmaf(fmaxf(__uint_as_float(v[k + 1]), nb[c0 + k + 1]), w2[c0 + k + 1], acc1);
+          }
+        }
+        part[set * 512 + r * 128 + px] = acc + acc1;
       }
+      ppar ^= 1;
       tc_before();
-      asm volatile("bar.sync %0, 128;\n" ::"r"(1 + set) : "memory");
+      __syncthreads();
+      const int e = set * 128 + px;   // row set of the group, column px
+      float* w = wout + ((size_t)b * 128 + y0 + 4 * g + set) * 128 + px;
+      const float sum = (part[e] + part[512 + e]) + (part[1024 + e] + part[1536 + e]);
+      *w = sum + (h0 == 0 ? net.b2 : *w);
+      __syncthreads();
     }
-    wout[((size_t)b * 128 + y0 + 4 * g + set) * 128 + px] = acc + net.b2;
   }
   tc_before();
   __syncthreads();
@@ -568,9 +718,9 @@ int pc_launch(const PinoClusterNet& net, const PinoState* st, float* wout, int B
 
 int launch_pino_cluster(const PinoClusterNet& net, const PinoState* st, float* wout, int B, int* err,
                         cudaStream_t s) {
-  // Clusters of 16 halve every stage's rows (one to seven states 56 us, against 76 with 8) while
-  // they all run at once; beyond that twice as many clusters of 8 fit (8 states: 76 us, against
-  // 112 in two waves of 16; 15 states 79).
+  // Clusters of 16 halve every stage's rows (one to seven states 48 us, against 62 with 8) while
+  // they all run at once; beyond that twice as many clusters of 8 fit (8 states: 62 us, against
+  // 96 in two waves of 16; 15 states 65).
   const int c16 = pc_capacity<16>(), c8 = pc_capacity<8>();
   if (c16 > 0 && (c8 == 0 || B <= c16)) return pc_launch<16>(net, st, wout, B, err, s);
   return pc_launch<8>(net, st, wout, B, err, s);
