@@ -497,9 +497,11 @@ __global__ void __launch_bounds__(kFineThreads, fine_blocks_per_sm(TC, TR)) fine
     }
     __syncwarp();
   };
-  // Inverse diagonals, by way of the private words: a rolled loop (executed once per launch, its
-  // unrolled code would be fetched at several clocks per instruction).
-#pragma unroll 1
+  // Inverse diagonals, by way of the private words: a loop of four pairs of nodes at a time (executed once
+  // per launch, its unrolled code would be fetched at several clocks per instruction; one
+  // pair at a time waits for each reciprocal: 32 slices of 1024 x 1024, 128 steps, 22.7 ms against
+  // 22.4).
+#pragma unroll 4
   for (int e = 0; e < TR * H; ++e) {
     const int r = e / H, i0 = col0 + e - r * H, i1 = i0 + H, j = row0 + r;
     const bool in = j >= 0 && j < M - 1;
