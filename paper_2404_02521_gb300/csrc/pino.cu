@@ -336,9 +336,9 @@ struct EpiProj { // P: rows pixels, cols hidden -> w = sum_h ReLU(v + b1) w2[h] 
 // CUDA-core kernels: restriction, lifting, prolongation + residual + far field (+ Parareal)
 // ---------------------------------------------------------------------------------------
 
-__global__ void pino_restrict_kernel(const PinoState* st, float* ump, int Mp) {
+__global__ void pino_restrict_kernel(const __grid_constant__ PinoStates st, float* ump, int Mp) {
   const int b = blockIdx.y;
-  const PinoState s = st[b];
+  const PinoState s = st.list ? st.list[b] : st.one;
   const size_t P = (size_t)Mp * Mp;
   const float ratio = (float)(s.M - 1) / (float)(Mp - 1);
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < P; e += (size_t)gridDim.x * blockDim.x) {
@@ -347,11 +347,11 @@ __global__ void pino_restrict_kernel(const PinoState* st, float* ump, int Mp) {
   }
 }
 
-__global__ void pino_lift_kernel(const PinoState* st, const float* ump, const float* lift_w,
+__global__ void pino_lift_kernel(const __grid_constant__ PinoStates st, const float* ump, const float* lift_w,
                                  const float* lift_b, bf16* act_cp, bf16* act_pc, int Mp, int C,
                                  int cin) {
   const int b = blockIdx.y;
-  const PinoState s = st[b];
+  const PinoState s = st.list ? st.list[b] : st.one;
   const size_t P = (size_t)Mp * Mp;
   const float hp = s.h * (float)(s.M - 1) / (float)(Mp - 1);   // network grid spacing
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < P; e += (size_t)gridDim.x * blockDim.x) {
@@ -381,9 +381,9 @@ struct ApplyArgs {
 //   PROP: out = G_new;  INIT: u_{n+1} = G_old = G_new;  ITER: u_{n+1} = F + (G_new - G_old),
 //   G_old = G_new;  ITER_SKIP: G_new = G_old (no network) and the ITER update.
 // Block partial sums (FP64, fixed order) of ||u_{n+1}||^2 and ||du||^2 per block.
-__global__ void pino_apply_kernel(const PinoState* st, const float* wout, int Mp, ApplyArgs aa) {
+__global__ void pino_apply_kernel(const __grid_constant__ PinoStates st, const float* wout, int Mp, ApplyArgs aa) {
   const int b = blockIdx.y;
-  const PinoState s = st[b];
+  const PinoState s = st.list ? st.list[b] : st.one;
   const int M = s.M;
   const size_t MM = (size_t)M * M, P = (size_t)Mp * Mp;
   const float ratio = (float)(Mp - 1) / (float)(M - 1);
@@ -468,7 +468,7 @@ __global__ void pino_defect_kernel(const double* partials, int nblocks, int pstr
 #define BS_TRY_LAUNCH(expr) do { cudaError_t e_ = (expr); if (e_ != cudaSuccess) return cuda_error(e_, #expr); } while (0)
 
 // the staged path: a 256 x 256 network grid, whose activations (4 MB) a cluster cannot hold
-static int pino_network256(bs_pino* net, PinoRes& R, const PinoState* st, int B, cudaStream_t s) {
+static int pino_network256(bs_pino* net, PinoRes& R, const PinoStates& st, int B, cudaStream_t s) {
   constexpr int Mp = 256, C = 32, mx = 12, MY = 24, P = Mp * Mp;
   const int pix_blocks = (P + 255) / 256;
   pino_lift_kernel<<<dim3(pix_blocks, B), 256, 0, s>>>(st, R.ump, net->lift_w, net->lift_b,
@@ -519,7 +519,7 @@ static PinoState make_state(const ItemDesc& d, const float* in, float* out, int 
 }
 
 // Network + residual for the states already in R.st (B of them), then the apply step.
-static int pino_run(bs_pino* net, PinoRes& R, const PinoState* st, int B, int Mmax,
+static int pino_run(bs_pino* net, PinoRes& R, const PinoStates& st, int B, int Mmax,
                     const ApplyArgs& aa, bool skip_net, cudaStream_t s) {
   const int Mp = R.Mp;
   if (!skip_net && Mp == 128) {
@@ -554,11 +554,10 @@ int pino_propagate(bs_pino* net, const bs_grid* g, const ItemDesc& d, const floa
   if (rc) return rc;
   PinoRes* R;
   if ((rc = ensure_res(net, network_grid(g->M), 1, 1, &R))) return rc;
-  PinoState st = make_state(d, in, out, g->M, g->xmax, tau0, dtau);
-  BS_CUDA_TRY(cudaMemcpyAsync(R->st, &st, sizeof(st), cudaMemcpyHostToDevice, s));
+  const PinoStates st = {nullptr, make_state(d, in, out, g->M, g->xmax, tau0, dtau)};
   ApplyArgs aa = {};
   aa.mode = PAPPLY_PROP;
-  return pino_run(net, *R, R->st, 1, g->M, aa, false, s);
+  return pino_run(net, *R, st, 1, g->M, aa, false, s);
 }
 
 // The PINO on B independent states at once (coarse_propagate_batched): one network launch
@@ -581,10 +580,12 @@ int pino_propagate_batched(bs_pino* net, const bs_grid* g, const ItemDesc* items
       sts[(size_t)i] = make_state(d, in[b0 + i], out[b0 + i], g->M, g->xmax, d.tau0, d.dtau);
     }
     // stream-ordered after the previous chunk's kernels, which read the descriptors
-    BS_CUDA_TRY(cudaMemcpyAsync(R->st, sts.data(), (size_t)nb * sizeof(PinoState), cudaMemcpyHostToDevice, s));
+    const PinoStates st = {nb > 1 ? R->st : nullptr, sts[0]};
+    if (nb > 1)
+      BS_CUDA_TRY(cudaMemcpyAsync(R->st, sts.data(), (size_t)nb * sizeof(PinoState), cudaMemcpyHostToDevice, s));
     ApplyArgs aa = {};
     aa.mode = PAPPLY_PROP;
-    if ((rc = pino_run(net, *R, R->st, nb, g->M, aa, false, s))) return rc;
+    if ((rc = pino_run(net, *R, st, nb, g->M, aa, false, s))) return rc;
   }
   return BS_OK;
 }
@@ -598,14 +599,9 @@ int pino_sweep(bs_pino* net, const bs_grid* g, const ItemDesc& d, const SweepArg
   const int M = g->M;
   const size_t MM = (size_t)M * M;
   PinoRes* R;
-  if ((rc = ensure_res(net, network_grid(M), 1, a.N, &R))) return rc;
+  if ((rc = ensure_res(net, network_grid(M), 1, 1, &R))) return rc;
   const int nblocks = (int)((MM + 255) / 256);
   const int pstride = 2 * nblocks;
-  // descriptors of all slices, uploaded once (slice n reads entry n)
-  std::vector<PinoState> sts((size_t)a.N);
-  for (int n = 0; n < a.N; ++n)
-    sts[(size_t)n] = make_state(d, a.U + (size_t)n * MM, nullptr, M, g->xmax, n * a.slice_len, a.slice_len);
-  BS_CUDA_TRY(cudaMemcpyAsync(R->st, sts.data(), sts.size() * sizeof(PinoState), cudaMemcpyHostToDevice, s));
   for (int n = a.n_first; n < a.N; ++n) {
     ApplyArgs aa;
     const bool skip = (a.mode == SWEEP_ITER && n == a.n_first);
@@ -614,7 +610,8 @@ int pino_sweep(bs_pino* net, const bs_grid* g, const ItemDesc& d, const SweepArg
     aa.Fn = a.Fb + (size_t)n * MM;
     aa.Gold = a.Gold + (size_t)n * MM;
     aa.partials = partials + (size_t)(n + 1) * pstride;
-    if ((rc = pino_run(net, *R, R->st + n, 1, M, aa, skip, s))) return rc;
+    const PinoStates st = {nullptr, make_state(d, a.U + (size_t)n * MM, nullptr, M, g->xmax, n * a.slice_len, a.slice_len)};
+    if ((rc = pino_run(net, *R, st, 1, M, aa, skip, s))) return rc;
   }
   const int n_lo = a.mode == SWEEP_INIT ? 1 : a.n_first + 1;
   pino_defect_kernel<<<1, 32, 0, s>>>(partials, nblocks, pstride, n_lo, a.N, a.n_first, a.norms,

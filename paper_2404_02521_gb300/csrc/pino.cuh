@@ -17,6 +17,13 @@ struct PinoState {
   PayoffF pf;
 };
 
+// The states of a launch: a device array, or (list NULL) one state in the launch's own parameters,
+// which needs no copy ahead of it (one 128 x 128 state 47.1 -> 45.1 us).
+struct PinoStates {
+  const PinoState* list;
+  PinoState one;
+};
+
 // bilinear sample of a node field on an Mi grid at fractional node index (ti, tj)
 __device__ __forceinline__ float bilinear(const float* u, int Mi, float tx, float ty) {
   int i0 = min((int)floorf(tx), Mi - 2), j0 = min((int)floorf(ty), Mi - 2);
@@ -52,7 +59,7 @@ inline size_t pino_mix_index(int l, int q, int kx, int c, int o, int ri) {
 }
 
 // The network on B states (128 x 128 network grid): wout[b][y][x], the increment.
-int launch_pino_cluster(const PinoClusterNet& net, const PinoState* st, float* wout, int B, int* err,
+int launch_pino_cluster(const PinoClusterNet& net, const PinoStates& st, float* wout, int B, int* err,
                         cudaStream_t s);
 
 }  // namespace bsp

@@ -182,7 +182,7 @@ __device__ __forceinline__ float bf_hi(uint32_t v) { return __uint_as_float(v & 
 
 template <int CL>
 __global__ void __launch_bounds__(kPcThreads, 1)
-pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const PinoState* __restrict__ st,
+pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const __grid_constant__ PinoStates st,
                     float* __restrict__ wout, int* err) {
   using F = PcCfg<CL>;
   constexpr int G = F::G, ROWS = F::ROWS;
@@ -194,7 +194,7 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const PinoState*
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, set = warp >> 2, quad = warp & 3;
   const int rank = blockIdx.x, b = blockIdx.y, y0 = rank * ROWS;
   const bool leader = quad == 0 && lane == 0;   // of the set
-  const PinoState s = st[b];
+  const PinoState s = st.list ? st.list[b] : st.one;
   bool ok = true;
   auto wait1 = [&](uint64_t* mb, uint32_t parity) {   // one thread
     if (ok && !mbar_wait(mb, parity)) {
@@ -705,7 +705,7 @@ int pc_capacity() {
 }
 
 template <int CL>
-int pc_launch(const PinoClusterNet& net, const PinoState* st, float* wout, int B, int* err, cudaStream_t s) {
+int pc_launch(const PinoClusterNet& net, const PinoStates& st, float* wout, int B, int* err, cudaStream_t s) {
   BS_CUDA_TRY(pc_attributes<CL>());
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
@@ -716,7 +716,7 @@ int pc_launch(const PinoClusterNet& net, const PinoState* st, float* wout, int B
 
 }  // namespace
 
-int launch_pino_cluster(const PinoClusterNet& net, const PinoState* st, float* wout, int B, int* err,
+int launch_pino_cluster(const PinoClusterNet& net, const PinoStates& st, float* wout, int B, int* err,
                         cudaStream_t s) {
   // Clusters of 16 halve every stage's rows (one to seven states 48 us, against 62 with 8) while
   // they all run at once; beyond that twice as many clusters of 8 fit (8 states: 62 us, against
