@@ -49,7 +49,7 @@ struct bs_pino {
   bsp::bf16* R;    // [L][MY*mx][64][64]
   bsp::bf16* Wpw;  // [L][C][C]  (o, c)
   float* pw_b;     // [L][C]
-  bsp::bf16* W1;   // [H][C]
+  bsp::bf16* W1;   // [H][C], zero rows up to 128 or 256 (b1 and w2 alike)
   float* b1;       // [H]
   float* w2;       // [H]
   float b2_c;      // b2 + sum of b1 w2
@@ -496,9 +496,13 @@ static int pino_network256(bs_pino* net, PinoRes& R, const PinoStates& st, int B
     BS_TRY_LAUNCH((launch_umma2<32, 32, 32>(dim3(P / 128, B), pw, EpiAct{R.act_cp, R.act_pc, net->pw_b + l * C, P, C},
                                             net->err, s)));
   }
-  BS_TRY_LAUNCH((launch_umma<128, 32>(dim3(P / 128, B), GemmA{R.act_pc, (long long)P * C, C, P, C},
-                                      GemmB{net->W1, 0, 0}, EpiProj{R.wout, net->b1, net->w2, net->b2, P},
-                                      net->err, s)));
+  // the hidden nodes, padded to a tile of 128 or 256 columns by zero weights
+  const GemmA act{R.act_pc, (long long)P * C, C, P, C};
+  const EpiProj proj{R.wout, net->b1, net->w2, net->b2, P};
+  if (net->H <= 128)
+    BS_TRY_LAUNCH((launch_umma<128, 32>(dim3(P / 128, B), act, GemmB{net->W1, 0, 0}, proj, net->err, s)));
+  else
+    BS_TRY_LAUNCH((launch_umma<256, 32>(dim3(P / 128, B), act, GemmB{net->W1, 0, 0}, proj, net->err, s)));
   return BS_OK;
 }
 
@@ -718,6 +722,10 @@ extern "C" int pino_load(const char* path, bs_pino** out) {
       return rc;
     }
   }
+  const size_t Hp = H <= 128 ? 128 : H <= 256 ? 256 : (size_t)H;
+  W1.resize(Hp * C, to_bf16(0));
+  p1b.resize(Hp, 0.f);
+  p2w.resize(Hp, 0.f);
   if ((rc = upload(&net->lift_w, lift_w)) || (rc = upload(&net->lift_b, lift_b)) ||
       (rc = upload(&net->R, R)) || (rc = upload(&net->Wpw, Wpw)) || (rc = upload(&net->pw_b, pw_b)) ||
       (rc = upload(&net->W1, W1)) || (rc = upload(&net->b1, p1b)) || (rc = upload(&net->w2, p2w)) ||

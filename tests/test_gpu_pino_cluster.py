@@ -1,5 +1,5 @@
-"""The PINO's cluster kernel: layer counts, hidden widths at and between its 128-column passes, ragged
-states, and the two cluster sizes, against the network in 64 bits with the kernel's BF16
+"""The PINO's network paths (the cluster kernel to 128 x 128, the staged one beyond): layer counts,
+hidden widths at and between their column passes, ragged states, and the two cluster sizes, against the network in 64 bits with the kernel's BF16
 rounding points."""
 import dataclasses
 
@@ -11,12 +11,10 @@ from tests.gpu_util import start_state, to_gpu, to_np
 
 pytestmark = pytest.mark.gpu
 
-MP = 128
-
-
 def rounded_network(u, xmax, tau, dtau, p, w):
     """The increment w on the network grid and, per node, the sum of magnitudes it cancels from."""
     import torch
+    MP = 128 if u.shape[0] <= 128 else 256
     r = lambda a: a.float().bfloat16().double()                                     # noqa: E731
     t = lambda a: torch.tensor(np.asarray(a), device="cuda").double()               # noqa: E731
     C, mx, my = 32, 12, 12
@@ -59,7 +57,8 @@ def rounded_network(u, xmax, tau, dtau, p, w):
     return h @ w2 + float(w["proj2_b"]), h @ w2.abs()
 
 
-@pytest.mark.parametrize("layers,hidden,M", [(1, 16, 128), (2, 144, 128), (3, 256, 41), (5, 128, 127), (1, 112, 8)])
+@pytest.mark.parametrize("layers,hidden,M", [(1, 16, 128), (2, 144, 128), (3, 256, 41), (5, 128, 127), (1, 112, 8),
+                                             (1, 16, 256), (2, 144, 200)])
 def test_shapes(tmp_path, layers, hidden, M):
     import torch
     import paper_2404_02521_gb300 as bs
@@ -82,6 +81,7 @@ def test_shapes(tmp_path, layers, hidden, M):
         torch.cuda.synchronize()
         assert torch.equal(one, outs[k])
         want, size = (v.cpu().numpy() for v in rounded_network(ins[k], 4.0, taus[k], 1.0 / 64, p, w))
+        MP = want.shape[0]
         if M != MP:
             pos = np.arange(M) * ((MP - 1) / (M - 1))
             i0 = np.minimum(np.floor(pos).astype(int), MP - 2)
