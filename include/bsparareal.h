@@ -192,8 +192,8 @@ int coarse_propagate(const bs_grid* g, int kind, const bs_pino* net, const bs_pa
  *  kind = BS_COARSE_NUM: one thread-block cluster per state, one launch per run of
  *    consecutive items with equal parameters (at most 64 states each); on a grid with a
  *    coarse grid (bs_grid_set_coarse) the states are propagated one after another.
- *  kind = BS_COARSE_PINO: the network on up to 128 states per launch chain (every GEMM of the
- *    chain carries the states as extra rows or grid blocks); nsteps is ignored.
+ *  kind = BS_COARSE_PINO: the network on up to 128 states per launch chain (M <= 128: a cluster per
+ *    state; else every product carries the states as extra rows or grid blocks); nsteps is ignored.
  * For concurrent solves or requests whose coarse steps are due together (a slice of each).
  * Results for an item do not depend on B or on the other items (bitwise).
  *  p[B], u_in[B], u_out[B], tau0[B]  host arrays (u_in/u_out: device float[M*M], may alias)

@@ -17,7 +17,7 @@
 // memory: 40 issued instructions per node-step.  Measured on a GB300 at 2070 MHz, before and
 // after: 64 states of 256 x 256, 512 steps, 14.1 -> 7.6 ms (the packed FP32 pipe 46% busy); one
 // such state 2.00 -> 0.88 ms; 8 states of 64 x 64, 256 steps, 0.67 -> 0.28 ms; 32 states of
-// 1024 x 1024, 1024 steps, 219 -> 174 ms.  What is left is latency: two warps per scheduler
+// 1024 x 1024, 1024 steps, 219 -> 171 ms.  What is left is latency: two warps per scheduler
 // leave the FP32 pipe idle while both load, shuffle or wait.
 //
 // Exchange.  A warp needs one row from the warp above and one from the warp below, each sweep.

@@ -9,20 +9,17 @@ workloads, one kernel each:
   fine256    F on all 64 slices of the 256x256 exchange workload, 512 steps (one launch)
   coarse256  the initial serial coarse sweep of that workload (64 slices x 4 BiCGSTAB steps)
   tile1024   F on 48 slices of a 1024x1024 basket grid, 40 steps of the large-solve step size
-             (temporally blocked cluster tiles; 48 x 4 MB of state exceeds the 129 MB L2).  The
-             launch plan of one call: the cold first step split over two launches, the warm
-             second step with the third, two extrapolated steps per launch up to step 14, then
-             four steps of five sweeps per launch (the twelfth launch, steps 23-26, is the
-             steady state of the large solve)
+             (regions of register tiles, several whole steps per launch; 48 x 4 MB of state exceeds
+             the 129 MB L2)
   solve256   one Parareal solve of that workload (rho = 0.7): payoff, initial coarse sweep,
              then per iteration the batched F launch and a correcting coarse sweep
-  coarse512  coarse propagation of one 512x512 state, 4 steps (global-memory BiCGSTAB)
+  coarse512  coarse propagation of one 512x512 state, 4 steps (the cooperative grid solver)
   large1024  the large single solve: basket on 1024x1024, N = 128 slices of 1024 fine steps,
              numerical G with 4 steps per slice on a 256x256 grid (bilinear resampling);
              prints Parareal time to tolerance, iterations and serial fine stepping time
   pino128    the PINO coarse propagator on 64 states of 128x128 (random weights)
   pino128b   the PINO on 128 states of 128x128 in one coarse_propagate_batched call (random
-             weights): the network's GEMM chain with the states as extra rows or blocks
+             weights): a cluster per state, nine waves
   resample1024  Parareal to K = N = 4 on 1024x1024 basket states with numerical G on the 256x256
              grid (bilinear restriction and prolongation kernels, 64 fine steps per slice)
   fine3_64   three-asset F: 16 states of 64^3 nodes, 64 implicit steps (19-point stencil)
