@@ -239,9 +239,11 @@ __device__ __forceinline__ void xround(Xchg& xs, const float (&v)[NV], float (&t
 
 // The quotients of the Krylov scalars, on the serial path of every iteration: 2 ulp and no
 // correction steps.  They need not be rounded: r, s and x follow whatever alpha and omega they are
-// given, and beta only sets the next direction.  (A divisor beyond 2^126 keeps the exact quotient.)
+// given, and beta only sets the next direction.  (A divisor that is subnormal or beyond 2^126 keeps the
+// rounded quotient: its reciprocal is out of range.)
 __device__ __forceinline__ float krylov_div(float a, float b) {
-  return fabsf(b) < 8.0e37f ? __fdividef(a, b) : a / b;
+  const float m = fabsf(b);
+  return m > 1.2e-38f && m < 8.0e37f ? __fdividef(a, b) : a / b;
 }
 
 // v with its sign flipped where bit k of `bits` is set: the product with the shadow residual
