@@ -52,7 +52,6 @@ struct bs_pino {
   bsp::bf16* W1;   // [H][C], zero rows up to 128 or 256 (b1 and w2 alike)
   float* b1;       // [H]
   float* w2;       // [H]
-  float b2_c;      // b2 + sum of b1 w2
   bsp::bf16 *mix, *Wpw_c, *W1_c;   // the cluster path's layouts of R, Wpw and W1 (pino.cuh); NULL for shapes it does not run
   float b2;
   int* err;
@@ -528,7 +527,7 @@ static int pino_run(bs_pino* net, PinoRes& R, const PinoStates& st, int B, int M
   const int Mp = R.Mp;
   if (!skip_net && Mp == 128) {
     const PinoClusterNet cn = {net->lift_w, net->lift_b, net->pw_b, net->b1, net->w2, R.Ex, R.Ey, R.Eyi,
-                               net->Wpw_c, net->W1_c, net->mix, net->b2_c, net->L, net->H};
+                               net->Wpw_c, net->W1_c, net->mix, net->b2, net->L, net->H};
     const int rc = launch_pino_cluster(cn, st, R.wout, B, net->err, s);
     if (rc) return rc;
   } else if (!skip_net) {
@@ -701,9 +700,6 @@ extern "C" int pino_load(const char* path, bs_pino** out) {
   int rc;
   if (C == 32 && mx == 12 && my == 12 && H % 16 == 0 && H <= 256) {
     std::vector<bf16> mix((size_t)L * MYx * 2 * C * C), wc;
-    double bw = p2b[0];
-    for (int h = 0; h < H; ++h) bw += (double)p1b[h] * p2w[h];
-    net->b2_c = (float)bw;
     for (int l = 0; l < L; ++l) {
       for (size_t m = 0; m < MYx; ++m)
         for (int c = 0; c < C; ++c)

@@ -46,7 +46,7 @@ struct PinoClusterNet {
   const bf16* pw;      // [L][32][32] canonical (o, c)
   const bf16* w1;      // [H][32] canonical
   const bf16* mix;     // [L][72][2][4][4][32][4][2]: mode matrices, see pino_mix_index
-  float b2;            // b2 + sum of b1 w2
+  float b2;
   int L, H;
 };
 

@@ -20,7 +20,7 @@
 // launches, activations through L2, 16k tiles of one MMA each per stage and scattered 2-byte
 // stores) and one state 170 us, nearly all of it launch and tile latency.  Here the tensor work
 // of a stage is a few dozen MMAs per CTA and the bound is the chain of stages: their epilogues and
-// three exchanges per layer: one state 48 us, 128 states 502 us (with the apply kernel).  Per layer at
+// three exchanges per layer: one state 45 us, 128 states 506 us (with the apply kernel).  Per layer at
 // CL = 8 (22 k cycles): MMAs 7.5 k (a 128 x N x 16 MMA takes 64 cycles and more at N = 32, the A tile's
 // fetch; the M-major ones 100), G3 3.6 k, exchanges 5 k, epilogues 4 k.
 //
@@ -603,7 +603,7 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const __grid_con
   // ---- projection, 128 hidden nodes at a time for the four rows of a group: each set takes 32 hidden
   // nodes, whose biases and weights it keeps in registers, and the sets' sums meet in shared
   // memory (with a set per row every bias and weight is a shared-memory or constant-bank read per
-  // row: 4200 and 4600 cycles per group, now 3600).  ReLU(v + b) w = max(v, -b) w + b w, the sum of b w in net.b2.
+  // row: 4200 and 4600 cycles per group, now 3600).
   wait(&bar.ldw, 0);
   float* part = reinterpret_cast<float*>(smem + F::YZ);   // [set][row][128]
   uint32_t ppar = 0;
@@ -611,11 +611,11 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const __grid_con
 #pragma unroll 1
   for (int h0 = 0; h0 < net.H; h0 += 128) {
     const int n = min(128, net.H - h0);
-    float nb[32], w2[32];
+    float b1[32], w2[32];
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
       const int h = set * 32 + k;
-      nb[k] = h < n ? -net.b1[h0 + h] : 0.f;
+      b1[k] = h < n ? net.b1[h0 + h] : 0.f;
       w2[k] = h < n ? net.w2[h0 + h] : 0.f;
     }
 #pragma unroll 1
@@ -642,8 +642,8 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const __grid_con
           pc_ld_wait();
 #pragma unroll
           for (int k = 0; k < 16; k += 2) {
-            acc = fmaf(fmaxf(__uint_as_float(v[k]), nb[c0 + k]), w2[c0 + k], acc);
-            acc1 = fmaf(fmaxf(__uint_as_float(v[k + 1]), nb[c0 + k + 1]), w2[c0 + k + 1], acc1);
+            acc = fmaf(fmaxf(__uint_as_float(v[k]) + b1[c0 + k], 0.f), w2[c0 + k], acc);
+            acc1 = fmaf(fmaxf(__uint_as_float(v[k + 1]) + b1[c0 + k + 1], 0.f), w2[c0 + k + 1], acc1);
           }
         }
         part[set * 512 + r * 128 + px] = acc + acc1;
@@ -718,7 +718,7 @@ int pc_launch(const PinoClusterNet& net, const PinoStates& st, float* wout, int 
 
 int launch_pino_cluster(const PinoClusterNet& net, const PinoStates& st, float* wout, int B, int* err,
                         cudaStream_t s) {
-  // Clusters of 16 halve every stage's rows (one to seven states 48 us, against 62 with 8) while
+  // Clusters of 16 halve every stage's rows (one state 45 us, seven 48, against 62 with 8) while
   // they all run at once; beyond that twice as many clusters of 8 fit (8 states: 62 us, against
   // 96 in two waves of 16; 15 states 65).
   const int c16 = pc_capacity<16>(), c8 = pc_capacity<8>();
