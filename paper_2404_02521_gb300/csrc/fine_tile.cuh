@@ -387,13 +387,15 @@ __global__ void __launch_bounds__(kFineThreads, fine_blocks_per_sm(TC, TR)) fine
   // The warp's own rows of (hi, lo, increment, previous increment) arrive in four staging planes by
   // asynchronous copies, coalesced along the row, all in flight at once; nodes outside the
   // domain are zero.  16-byte copies where the grid and the input allow them (a chunk then lies
-  // wholly inside or outside), else 4-byte ones.  Chunks of four columns are swizzled, so that
+  // wholly inside or outside), else 4-byte ones.  A copy that only fills zeros names the plane's
+  // own array: the source has to be aligned to the copy even where nothing is read.  Chunks of four columns are swizzled, so that
   // a lane reads its columns of a row as whole chunks without bank conflicts.
   auto plane_at = [](int r, int c) { return r * W + (((c >> 2) ^ ((c >> 5) & 1)) << 2) + (c & 3); };
   float* plane = reinterpret_cast<float*>(smem + L::S0) + warp * TR * W;   // the warp's rows of the first plane
   {
     const float* ws = fb.ws + (size_t)blockIdx.z * 8 * MM + (size_t)(fl.par * 4) * MM;
     const bool vec = M % 4 == 0 && (!fl.first || (uintptr_t)d.in % 16 == 0);
+    const float* nowhere = fl.first ? d.in : fb.ws;
     auto load = [&](float* dst, const float* g) {   // g: the plane at this warp's first row and the region's first column
       if (vec) {
 #pragma unroll
@@ -402,7 +404,7 @@ __global__ void __launch_bounds__(kFineThreads, fine_blocks_per_sm(TC, TR)) fine
           for (int q = 0; q < (W + 127) / 128; ++q) {
             const int c = 4 * lane + 128 * q, i = ix0 + c, j = row0 + r;
             const bool in = c < W && i >= 0 && i < M && j >= 0 && j < M;
-            if (c < W) cp_async16(dst + plane_at(r, c), in ? g + (long long)r * M + c : fb.it[0].in, in);
+            if (c < W) cp_async16(dst + plane_at(r, c), in ? g + (long long)r * M + c : nowhere, in);
           }
       } else {
 #pragma unroll
@@ -411,7 +413,7 @@ __global__ void __launch_bounds__(kFineThreads, fine_blocks_per_sm(TC, TR)) fine
           for (int q = 0; q < TC; ++q) {
             const int c = lane + 32 * q, i = ix0 + c, j = row0 + r;
             const bool in = i >= 0 && i < M && j >= 0 && j < M;
-            cp_async4(dst + plane_at(r, c), in ? g + (long long)r * M + c : fb.it[0].in, in);
+            cp_async4(dst + plane_at(r, c), in ? g + (long long)r * M + c : nowhere, in);
           }
       }
     };
