@@ -16,6 +16,13 @@ namespace bsp {
 constexpr int kGridPolls = 1 << 22;      // bound on the polls of one barrier
 constexpr int kGridMaxBlocks = 1024;     // blocks of a group, as sized in the partial sums
 
+// Whether a counter that only grows has reached the target.  Both are taken modulo 2^32 (a launch of
+// 150 blocks passes that in 28 million barriers, minutes of iterations), and a counter is never
+// 2^31 away from a target that a block waits for.
+__host__ __device__ __forceinline__ bool grid_reached(unsigned seen, unsigned target) {
+  return (int)(seen - target) >= 0;
+}
+
 struct GridWords {
   float4 partials[2][kGridMaxBlocks];
   unsigned arrivals;   // zero at launch
@@ -43,7 +50,7 @@ struct GridGroup {
       unsigned seen = 0;
       while (true) {
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(seen) : "l"(&words->arrivals) : "memory");
-        if (seen >= target) break;
+        if (grid_reached(seen, target)) break;
         if (++polls >= kGridPolls || ((polls & 1023) == 0 && (*(volatile int*)status & 2))) {
           atomicOr(status, 2);
           out = 1;
