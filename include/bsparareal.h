@@ -278,7 +278,8 @@ int bs_fine_sweeps(const bs_grid* g, const bs_params* p, double dtau, int first_
 
 /* Solver options (process-wide; set them before launching work, not concurrently with it).
  *  BS_OPT_FINE_SWEEPS    Jacobi sweeps per fine step, >= 2; 0 = derive from the contraction
- *                        bound (default)
+ *                        bound (default).  Where extrapolated starts would not converge with a
+ *                        forced count, every step starts from the previous increment
  *  BS_OPT_JACOBI_TARGET  the derived sweep count of a warm-started step (each step starts
  *                        from the previous step's increment) makes q^sweeps <= this
  *                        (default 2^-10)
@@ -297,7 +298,9 @@ int bs_fine_sweeps(const bs_grid* g, const bs_params* p, double dtau, int first_
  *  BS_OPT_JACOBI_TARGET_EXTRAP_LATE  the extrapolated-start target from BS_OPT_EXTRAP_LATE on
  *                        (default 0.5: two sweeps, the structural minimum, wherever q <= 0.707;
  *                        at the 1024 x 1024 large-solve step, q = 0.63, the error against the FP64
- *                        oracle after 1024 steps is 6e-8 max|V| with two, three or five sweeps)
+ *                        oracle after 1024 steps is 6e-8 max|V| with two, three or five sweeps).
+ *                        Extrapolated starts converge with an even count, or where q^sweeps <= 1/3:
+ *                        the derived count is raised to the next one that does
  *  BS_OPT_PIPELINE       1 (default): parareal_solve with the numerical G (on the state grid
  *                        or on a coarse grid) and N >= 8 splits each coarse sweep into chunks
  *                        of consecutive slices (as many as F runs in one wave beside the

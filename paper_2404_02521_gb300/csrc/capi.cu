@@ -1,5 +1,6 @@
 // C ABI of the Black-Scholes Parareal library: handles, argument checks, the payoff kernel
 // (K6) and the Parareal driver loop (eq. parareal, Sec. 3.1).
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdarg>
@@ -80,10 +81,48 @@ double jacobi_contraction(int M, const bs_params& p, double dtau) {
   return q;
 }
 
+// A bound of |Im l| over the eigenvalues l of the Jacobi sweep: the largest row sum of the skew part of
+// D^{-1/2} (off-diagonal part) D^{-1/2}.  Neighbours' weights differ by (2i + 1)(r - sigma^2) dtau / 2
+// along an axis and by at most (i + j + 1) |rho| sigma1 sigma2 dtau / 4 across it, and a diagonal is at
+// least its own axis's part; each axis is maximised by itself.
+double jacobi_skew(int M, const bs_params& p, double dtau) {
+  const double g = 0.25 * std::fabs(p.rho) * p.sigma1 * p.sigma2 * dtau;
+  double bound = g;
+  for (const double sigma : {p.sigma1, p.sigma2}) {
+    const double a = 0.5 * sigma * sigma * dtau, c = std::fabs(0.5 * p.r * dtau - a) + g;
+    double s = c;
+    for (int i = 1; i <= M - 2; ++i) s = std::fmax(s, 2.0 * i * c / (1.0 + 2.0 * a * (i - 1.0) * (i - 1.0)));
+    bound += s;
+  }
+  return bound;
+}
+
 Options g_opt;
 
+// The error of an extrapolated start followed by m sweeps obeys e_{t+1} = l^m (2 e_t - e_{t-1}) for an
+// eigenvalue l of the sweep, whose roots z^2 = 2 a z - a (a = l^m) lie inside the unit circle where
+// |a| <= 1/3, and beyond that where a lies closer to the positive axis than the curve
+// a = z^2 / (2 z - 1), |z| = 1.  |l| <= q and |Im l| <= skew, so an even count keeps a within the
+// angle m asin(skew / |l|) of that axis; the bound on skew asks for half of what the curve's angle
+// at |a| = q^m allows.  (An odd count with rho = 0 and q = 0.75, or two sweeps with drift well above
+// diffusion, lost every digit within 100 steps.)
+bool extrap_stable(double q, double skew, int m) {
+  const double a = std::pow(q, m);
+  if (a <= 1.0 / 3.0) return true;
+  if (m % 2 != 0 || !(a < 1.0)) return false;
+  const double phi = std::acos((5.0 - 1.0 / (a * a)) / 4.0);   // |z^2 / (2 z - 1)| = 1 / sqrt(5 - 4 cos phi)
+  const double psi = 2.0 * phi - std::atan2(2.0 * std::sin(phi), 2.0 * std::cos(phi) - 1.0);
+  return skew <= 0.5 * std::pow(1.0 / 3.0, 1.0 / m) * std::sin(psi / m);
+}
+
+int extrap_sweeps(double q, double skew, int m) {
+  if (extrap_stable(q, skew, m)) return m;
+  if (extrap_stable(q, skew, m + 1)) return m + 1;
+  return std::max(m, (int)std::ceil(std::log(1.0 / 3.0) / std::log(q)));
+}
+
 // Sweeps so that q^m <= target (at least 2: the first sweep forms b, the last applies d).
-int sweeps_for(double q, int start) {
+int sweeps_for(double q, double skew, int start) {
   if (!(q < 0.8)) return 0;
   if (g_opt.fine_sweeps > 0) return g_opt.fine_sweeps;
   if (q <= 0.0) return 2;
@@ -91,8 +130,22 @@ int sweeps_for(double q, int start) {
                         : start == START_EXTRAP      ? g_opt.jacobi_target_extrap
                         : start == START_EXTRAP_LATE ? g_opt.jacobi_target_extrap_late
                                                      : g_opt.jacobi_target;
-  int m = (int)std::ceil(std::log(target) / std::log(q));
-  return m < 2 ? 2 : m;
+  const int m = std::max(2, (int)std::ceil(std::log(target) / std::log(q)));
+  return start == START_EXTRAP || start == START_EXTRAP_LATE ? extrap_sweeps(q, skew, m) : m;
+}
+
+FineCounts fine_counts(double q, double skew) {
+  FineCounts c;
+  c.sweeps = sweeps_for(q, skew, START_WARM);
+  c.sweeps0 = sweeps_for(q, skew, START_COLD);
+  c.sweepsx = sweeps_for(q, skew, START_EXTRAP);
+  c.sweepsxl = sweeps_for(q, skew, START_EXTRAP_LATE);
+  c.xstart = g_opt.extrap_start;
+  c.xlate = std::max(g_opt.extrap_late, g_opt.extrap_start);
+  // a forced count that extrapolated starts do not converge with: every step starts from the previous
+  // increment
+  if (c.sweeps > 0 && g_opt.fine_sweeps > 0 && !extrap_stable(q, skew, g_opt.fine_sweeps)) c.xstart = c.xlate = 1 << 30;
+  return c;
 }
 
 // Band shapes of the cluster-resident kernels (NCOL columns, NT threads, K rows per thread,
@@ -144,13 +197,14 @@ int launch_payoff(const bs_grid* g, const ItemDesc& d, float* u, cudaStream_t s)
   return BS_OK;
 }
 
-int grid_sweeps(bs_grid* g, const bs_params& p, double dtau, int start) {
+FineCounts grid_counts(bs_grid* g, const bs_params& p, double dtau) {
   const double key[6] = {p.sigma1, p.sigma2, p.rho, p.r, dtau, (double)g->M};
   if (std::memcmp(key, g->q_key, sizeof(key)) != 0) {
     g->q_val = jacobi_contraction(g->M, p, dtau);
+    g->q_skew = jacobi_skew(g->M, p, dtau);
     std::memcpy(g->q_key, key, sizeof(key));
   }
-  return sweeps_for(g->q_val, start);
+  return fine_counts(g->q_val, g->q_skew);
 }
 
 // Fine propagation of items whose Jacobi bound is too large for the sweep steppers: every
@@ -217,7 +271,7 @@ int bs_grid_create(int M, double xmax, bs_grid** out) {
   g->xmax = xmax;
   g->shape = band_shape(M);
   std::memset(g->q_key, 0, sizeof(g->q_key));
-  g->q_val = 0.0;
+  g->q_val = g->q_skew = 0.0;
   cudaError_t e = cudaGetDevice(&g->device);
   note_device_alloc();
   note_device_alloc();
@@ -259,7 +313,9 @@ int bs_payoff(const bs_grid* g, const bs_params* p, float* u, bs_stream stream) 
 int bs_fine_sweeps(const bs_grid* g, const bs_params* p, double dtau, int first_step) {
   if (!g || check_params(p) || !(dtau > 0.0)) return 0;
   if (first_step < 0 || first_step > 3) return 0;
-  return grid_sweeps(const_cast<bs_grid*>(g), *p, dtau, first_step);
+  const FineCounts c = grid_counts(const_cast<bs_grid*>(g), *p, dtau);
+  const int by_start[] = {c.sweeps, c.sweeps0, c.sweepsx, c.sweepsxl};   // in the order of SweepStart
+  return by_start[first_step];
 }
 
 int fine_propagate_batched(const bs_grid* g, const bs_params* p, const float* const* u_in,
@@ -277,10 +333,7 @@ int fine_propagate_batched(const bs_grid* g, const bs_params* p, const float* co
     ItemDesc d = make_item(p[b], tau0[b], dtau[b]);
     d.in = u_in[b];
     d.out = u_out[b];
-    d.sweeps = grid_sweeps(const_cast<bs_grid*>(g), p[b], dtau[b]);
-    d.sweeps0 = grid_sweeps(const_cast<bs_grid*>(g), p[b], dtau[b], START_COLD);
-    d.sweepsx = grid_sweeps(const_cast<bs_grid*>(g), p[b], dtau[b], START_EXTRAP);
-    d.sweepsxl = grid_sweeps(const_cast<bs_grid*>(g), p[b], dtau[b], START_EXTRAP_LATE);
+    set_counts(d, grid_counts(const_cast<bs_grid*>(g), p[b], dtau[b]));
     items[(size_t)b] = d;
   }
   cudaStream_t s = (cudaStream_t)stream;
@@ -631,11 +684,8 @@ int parareal_solve(const bs_grid* gc, const bs_params* p, int N, int fine_steps,
   const size_t MM = (size_t)M * M;
   const double slice = p->T / N;
   const double dtau_f = slice / fine_steps;
-  const int sweeps = grid_sweeps(g, *p, dtau_f);
-  const int sweeps0 = grid_sweeps(g, *p, dtau_f, START_COLD);
-  const int sweepsx = grid_sweeps(g, *p, dtau_f, START_EXTRAP);
-  const int sweepsxl = grid_sweeps(g, *p, dtau_f, START_EXTRAP_LATE);
-  const bool krylov_f = sweeps == 0;   // Jacobi bound >= 0.8: F by BiCGSTAB per step
+  const FineCounts counts = grid_counts(g, *p, dtau_f);
+  const bool krylov_f = counts.sweeps == 0;   // Jacobi bound >= 0.8: F by BiCGSTAB per step
   // numerical G on this grid: F overlapped with the chunked coarse sweep (Krylov F of grids
   // beyond one cluster shares the coarse solver's global workspace and stays sequential)
   if (!pino && g_opt.pipeline && pipeline_eligible(N) && !(krylov_f && g->M > 256))
@@ -713,10 +763,7 @@ int parareal_solve(const bs_grid* gc, const bs_params* p, int N, int fine_steps,
       ItemDesc d = make_item(*p, n * slice, dtau_f);
       d.in = u_out + (size_t)n * MM;
       d.out = Fb + (size_t)n * MM;
-      d.sweeps = sweeps;
-      d.sweeps0 = sweeps0;
-      d.sweepsx = sweepsx;
-      d.sweepsxl = sweepsxl;
+      set_counts(d, counts);
       items[(size_t)(n - k)] = d;
     }
     if ((rc = tf.begin(s))) return rc;

@@ -195,7 +195,26 @@ enum SweepStart { START_WARM = 0, START_COLD = 1, START_EXTRAP = 2, START_EXTRAP
 __host__ __device__ inline int step_sweeps(const ItemDesc& d, int step) {
   return step == 0 ? d.sweeps0 : step < d.xstart ? d.sweeps : step < d.xlate ? d.sweepsx : d.sweepsxl;
 }
-int sweeps_for(double q, int start);
+int sweeps_for(double q, double skew, int start);
+double jacobi_skew(int M, const bs_params& p, double dtau);
+
+// How F solves its steps: the Jacobi sweeps of a step by its start (as in ItemDesc).
+struct FineCounts {
+  int sweeps, sweeps0, sweepsx, sweepsxl, xstart, xlate;   // sweeps 0: the Jacobi bound is too large
+};
+FineCounts fine_counts(double q, double skew);
+inline void set_counts(ItemDesc& d, const FineCounts& c) {
+  d.sweeps = c.sweeps;
+  d.sweeps0 = c.sweeps0;
+  d.sweepsx = c.sweepsx;
+  d.sweepsxl = c.sweepsxl;
+  d.xstart = c.xstart;
+  d.xlate = c.xlate;
+}
+// Whether extrapolated starts followed by m sweeps converge, and the least count from m on with
+// which they do (capi.cu).
+bool extrap_stable(double q, double skew, int m);
+int extrap_sweeps(double q, double skew, int m);
 BandShape band_shape(int M);
 
 struct Options {
@@ -253,7 +272,7 @@ struct bs_grid {
   void* pipe = nullptr;        // pipelined driver: second stream and events (pipeline.cu)
   // cached contraction
   double q_key[6];
-  double q_val;
+  double q_val, q_skew;
   // phase accounting (bs_phase_stats)
   double ms_fine = 0.0, ms_coarse = 0.0;
   int n_fine = 0, n_coarse = 0, n_other = 0;
@@ -264,8 +283,8 @@ namespace bsp {
 int launch_fine(const bs_grid* g, const ItemDesc* items, int n, int nsteps, cudaStream_t s);
 int fine_launches(const bs_grid* g, const ItemDesc* items, int n, int nsteps);   // kernels launch_fine enqueues
 int launch_payoff(const bs_grid* g, const ItemDesc& d, float* u, cudaStream_t s);
-// Jacobi sweeps per fine step on this grid (cached contraction bound; 0 if q >= 0.8)
-int grid_sweeps(bs_grid* g, const bs_params& p, double dtau, int start = START_WARM);
+// Jacobi sweeps of F's steps on this grid (cached contraction bound; 0 if q >= 0.8)
+FineCounts grid_counts(bs_grid* g, const bs_params& p, double dtau);
 // Coarse numerical propagation / Parareal serial sweep (see coarse.cu).
 enum { SWEEP_PROP = 0, SWEEP_INIT = 1, SWEEP_ITER = 2 };
 // Independent states propagated by one batched SWEEP_PROP launch (one cluster each): the

@@ -76,9 +76,8 @@ extern "C" int parareal_solve_noalloc(int M, double xmax, const bs_params* p, in
   const double slice = p->T / N;
   const double dtau_f = slice / fine_steps;
   const double q = jacobi_contraction(M, *p, dtau_f);
-  const int sweeps = sweeps_for(q, START_WARM), sweeps0 = sweeps_for(q, START_COLD);
-  const int sweepsx = sweeps_for(q, START_EXTRAP), sweepsxl = sweeps_for(q, START_EXTRAP_LATE);
-  if (sweeps == 0)
+  const FineCounts counts = fine_counts(q, jacobi_skew(M, *p, dtau_f));
+  if (counts.sweeps == 0)
     return set_error(BS_ERR_ARG,
                      "parareal_solve_noalloc: the fine step's Jacobi bound %.3f is >= 0.8 (only the "
                      "Jacobi stepper runs without allocation); use more fine steps or parareal_solve", q);
@@ -136,10 +135,7 @@ extern "C" int parareal_solve_noalloc(int M, double xmax, const bs_params* p, in
         ItemDesc d = make_item(*p, n * slice, dtau_f);
         d.in = u_out + (size_t)n * MM;
         d.out = Fb + (size_t)n * MM;
-        d.sweeps = sweeps;
-        d.sweeps0 = sweeps0;
-        d.sweepsx = sweepsx;
-        d.sweepsxl = sweepsxl;
+        set_counts(d, counts);
         items[i] = d;
       }
       if ((rc = launch_fine(&g, items, B, fine_steps, s))) return rc;

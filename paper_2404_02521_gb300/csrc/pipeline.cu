@@ -119,11 +119,8 @@ int parareal_pipelined(bs_grid* g, const bs_params* p, int N, int fine_steps, in
   const size_t MM = (size_t)M * M;
   const double slice = p->T / N;
   const double dtau_f = slice / fine_steps;
-  const int sweeps = grid_sweeps(g, *p, dtau_f);
-  const int sweeps0 = grid_sweeps(g, *p, dtau_f, START_COLD);
-  const int sweepsx = grid_sweeps(g, *p, dtau_f, START_EXTRAP);
-  const int sweepsxl = grid_sweeps(g, *p, dtau_f, START_EXTRAP_LATE);
-  const bool krylov_f = sweeps == 0;
+  const FineCounts counts = grid_counts(g, *p, dtau_f);
+  const bool krylov_f = counts.sweeps == 0;
   const bool resampled = g->coarse_M > 0 && g->coarse_M != g->M;
   const bool cheap_f = g->shape.C >= 1 && g->shape.C <= kMaxCluster;   // a state per cluster
   const ItemDesc dc = make_item(*p, 0.0, slice / coarse_steps);
@@ -224,10 +221,7 @@ int parareal_pipelined(bs_grid* g, const bs_params* p, int N, int fine_steps, in
         // u_{cS} is rewritten by this iteration's sweep chunk c-1 while k < cS
         d.in = (n == c * S && c >= 1 && k < n) ? snap_at(k & 1, c) : u_out + (size_t)n * MM;
         d.out = Fb + (size_t)n * MM;
-        d.sweeps = sweeps;
-        d.sweeps0 = sweeps0;
-        d.sweepsx = sweepsx;
-        d.sweepsxl = sweepsxl;
+        set_counts(d, counts);
         items.push_back(d);
       }
       cudaEvent_t t0 = nullptr, t1 = nullptr;

@@ -94,7 +94,8 @@ struct Slot {
   float *U = nullptr, *Fb = nullptr, *Gold = nullptr;
   double* norms = nullptr;
   double* partials = nullptr;    // PINO requests: the sweep's defect partials
-  int k = 0, sweeps = 0, sweeps0 = 0, sweepsx = 0, sweepsxl = 0, result = BS_OK;
+  int k = 0, result = BS_OK;
+  FineCounts counts = {};
   double defect = 0.0, t_submit = 0.0;
 };
 
@@ -249,10 +250,7 @@ static int admit(bs_server* sv, Slot& sl, long long id, const bs_request& r, dou
   if ((rc = bs_grid_set_coarse(sl.g, r.coarse_kind == BS_COARSE_NUM ? r.coarse_M : 0))) return rc;
   const double slice = r.p.T / r.N;
   const double dtau_f = slice / r.fine_steps;
-  sl.sweeps = grid_sweeps(sl.g, r.p, dtau_f, START_WARM);
-  sl.sweeps0 = grid_sweeps(sl.g, r.p, dtau_f, START_COLD);
-  sl.sweepsx = grid_sweeps(sl.g, r.p, dtau_f, START_EXTRAP);
-  sl.sweepsxl = grid_sweeps(sl.g, r.p, dtau_f, START_EXTRAP_LATE);
+  sl.counts = grid_counts(sl.g, r.p, dtau_f);
   BS_CUDA_TRY(cudaMemsetAsync(sl.g->status, 0, kStatusWords * sizeof(int), sl.st));
   const ItemDesc dc = make_item(r.p, 0.0, slice / r.coarse_steps);
   if ((rc = launch_payoff(sl.g, dc, sl.U, sl.st))) return rc;
@@ -314,10 +312,7 @@ static int launch_group(bs_server* sv, const std::vector<Slot*>& grp) {
       ItemDesc d = make_item(sl->r.p, n * slice, slice / fs);
       d.in = sl->U + (size_t)n * MM;
       d.out = sl->Fb + (size_t)n * MM;
-      d.sweeps = sl->sweeps;
-      d.sweeps0 = sl->sweeps0;
-      d.sweepsx = sl->sweepsx;
-      d.sweepsxl = sl->sweepsxl;
+      set_counts(d, sl->counts);
       items.push_back(d);
     }
   }
