@@ -197,6 +197,25 @@ static double f3_contraction_scan(int M, const bs_params3& p, double dtau) {
   return q;
 }
 
+// jacobi_skew (capi.cu) for three assets.
+static double f3_skew(int M, const bs_params3& p, double dtau) {
+  const int pair[3][2] = {{0, 1}, {0, 2}, {1, 2}};
+  double cross[3] = {0.0, 0.0, 0.0}, bound = 0.0;
+  for (int c = 0; c < 3; ++c) {
+    const double g = 0.25 * std::fabs(p.rho[c]) * p.sigma[pair[c][0]] * p.sigma[pair[c][1]] * dtau;
+    cross[pair[c][0]] += g;
+    cross[pair[c][1]] += g;
+    bound += g;
+  }
+  for (int x = 0; x < 3; ++x) {
+    const double a = 0.5 * p.sigma[x] * p.sigma[x] * dtau, c = std::fabs(0.5 * p.r * dtau - a) + cross[x];
+    double s = c;
+    for (int i = 1; i <= M - 2; ++i) s = std::fmax(s, 2.0 * i * c / (1.0 + 2.0 * a * (i - 1.0) * (i - 1.0)));
+    bound += s;
+  }
+  return bound;
+}
+
 // The scan visits (M-1)^3 nodes (milliseconds at 128^3), and parareal_solve3 asks for the same
 // bound on every F call: the last few results are kept per (M, parameters, dtau).
 double f3_contraction(int M, const bs_params3& p, double dtau) {
@@ -231,14 +250,16 @@ double f3_contraction(int M, const bs_params3& p, double dtau) {
 // takes an even count: the error recurrence e_{t+1} = l^m (2 e_t - e_{t-1}) of an extrapolated
 // start has a root beyond 1 where l^m < -1/3 (l an eigenvalue of the sweep, which can be
 // negative).
+// Complex eigenvalues (drift above diffusion; skew bounds their imaginary part) need more, see
+// extrap_stable.
 constexpr int kF3ExtrapStart = 2;
-static int f3_sweeps(double q, int step) {
+static int f3_sweeps(double q, double skew, int step) {
   const double target = step == 0               ? 1.0 / 4194304.0
                         : step < kF3ExtrapStart ? 1.0 / 1024.0
                                                 : std::fmin(step / 128.0, 0.5);
   if (q <= 0.0) return 2;
   const int m = std::max(2, (int)std::ceil(std::log(target) / std::log(q)));
-  return target > 0.25 ? (m + 1) & ~1 : m;
+  return step < kF3ExtrapStart ? m : extrap_sweeps(q, skew, target > 0.25 ? (m + 1) & ~1 : m);
 }
 
 int f3_check(int M, double xmax, const bs_params3* p) {
@@ -326,6 +347,7 @@ int fine_propagate3(int M, double xmax, const bs_params3* p, const float* const*
   const double q = f3_contraction(M, *p, dtau);
   if (!(q < 0.8))
     return set_error(BS_ERR_ARG, "fine_propagate3: Jacobi bound %.3f >= 0.8 (take smaller steps)", q);
+  const double skew = f3_skew(M, *p, dtau);
   cudaStream_t s = (cudaStream_t)stream;
   const size_t n3 = (size_t)M * M * M;
   const unsigned blocks = (unsigned)((n3 + kF3Threads - 1) / kF3Threads);
@@ -357,7 +379,7 @@ int fine_propagate3(int M, double xmax, const bs_params3* p, const float* const*
     f3_phase_kernel<<<grid, kF3Threads, 0, s>>>(fb, F3_INIT, nsteps);
     int cur = 0;   // 0: the increment is in dA
     for (int step = 0; step < nsteps; ++step) {
-      const int m = f3_sweeps(q, step);   // >= 2
+      const int m = f3_sweeps(q, skew, step);   // >= 2
       for (int sw = 0; sw < m; ++sw) {
         const int face_step = step + 1 < nsteps ? step + 1 : -1;
         if (sw == 0)
