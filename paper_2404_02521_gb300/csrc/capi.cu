@@ -178,6 +178,23 @@ int ensure(Workspace& w, size_t bytes) {
   return BS_OK;
 }
 
+// A solve counts its own Krylov iterations.  Word 0 stays: a failure of an asynchronous call before it
+// is this call's to report.
+int begin_status(bs_grid* g, cudaStream_t s) {
+  g->failed = 0;
+  BS_CUDA_TRY(cudaMemsetAsync(g->status + 1, 0, (kStatusWords - 1) * sizeof(int), s));
+  return BS_OK;
+}
+
+// Clears the reported bits, so that the next call reports only what comes after them, and keeps them
+// for bs_grid_stats.
+int report_status(bs_grid* g, int bits, cudaStream_t s) {
+  g->failed = bits;
+  BS_CUDA_TRY(cudaMemsetAsync(g->status, 0, sizeof(int), s));
+  BS_CUDA_TRY(cudaStreamSynchronize(s));
+  return BS_OK;
+}
+
 __global__ void payoff_kernel(PayoffF pf, float* u, int M, float h) {
   const size_t n = (size_t)M * M;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n;
@@ -575,7 +592,8 @@ int bs_grid_stats(bs_grid* g, int* krylov_iters_max, int* krylov_failed, int* kr
   BS_CUDA_TRY(cudaMemcpy(h, g->status, kStatusWords * sizeof(int), cudaMemcpyDeviceToHost));
   BS_CUDA_TRY(cudaMemset(g->status, 0, kStatusWords * sizeof(int)));
   if (krylov_iters_max) *krylov_iters_max = h[1];
-  if (krylov_failed) *krylov_failed = h[0];   // bit 0: iteration cap, bit 1: exchange timeout
+  if (krylov_failed) *krylov_failed = h[0] | g->failed;   // bit 0: iteration cap, bit 1: exchange timeout
+  g->failed = 0;
   if (krylov_iters_total) *krylov_iters_total = h[2];
   if (krylov_solves) *krylov_solves = h[3];
   return BS_OK;
@@ -719,7 +737,7 @@ int parareal_solve(const bs_grid* gc, const bs_params* p, int N, int fine_steps,
     g->n_coarse += 1;
     return pino_sweep(pnet, g, d, sa, partials, s);
   };
-  BS_CUDA_TRY(cudaMemsetAsync(g->status, 0, kStatusWords * sizeof(int), s));
+  if ((rc = begin_status(g, s))) return rc;
   PhaseTimer tf, tc;
   tf.on = tc.on = g_opt.phase_timing != 0;
 
@@ -798,6 +816,7 @@ int parareal_solve(const bs_grid* gc, const bs_params* p, int N, int fine_steps,
       *k_done = k + 1;
       g->ms_fine += ms_f;
       g->ms_coarse += ms_c;
+      if ((rc = report_status(g, hstat, s))) return rc;
       if (hstat & 2)
         return set_error(BS_ERR_CUDA, "parareal_solve: a cluster exchange timed out");
       return set_error(BS_ERR_NOCONV, "parareal_solve: a coarse BiCGSTAB solve hit its iteration cap");

@@ -1074,8 +1074,10 @@ int coarse_autotune(bs_grid* g, const ItemDesc& d, cudaStream_t s, int steps, in
   float best_ms = 1e30f;
   int rc = BS_OK;
   note_device_alloc();
-  if (cudaMalloc(&buf, 2 * MM * sizeof(float)) != cudaSuccess || cudaEventCreate(&e0) != cudaSuccess ||
-      cudaEventCreate(&e1) != cudaSuccess) {
+  // two states, and status words of its own: the tuning solves' counts and failures are not the caller's
+  if (cudaMalloc(&buf, 2 * MM * sizeof(float) + kStatusWords * sizeof(int)) != cudaSuccess ||
+      cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess ||
+      cudaMemsetAsync(buf + 2 * MM, 0, kStatusWords * sizeof(int), s) != cudaSuccess) {
     rc = cuda_error(cudaGetLastError(), "coarse_autotune");
   }
   if (rc == BS_OK) rc = launch_payoff(g, d, buf, s);
@@ -1090,7 +1092,7 @@ int coarse_autotune(bs_grid* g, const ItemDesc& d, cudaStream_t s, int steps, in
     sp.a.csteps = steps;
     sp.a.in = buf;
     sp.a.out = buf + MM;
-    sp.a.status = g->status;
+    sp.a.status = reinterpret_cast<int*>(buf + 2 * MM);
     sp.a.tol = g_opt.krylov_tol;
     sp.a.maxit = g_opt.krylov_maxit;
     sp.sh.M = M;
@@ -1115,9 +1117,6 @@ int coarse_autotune(bs_grid* g, const ItemDesc& d, cudaStream_t s, int steps, in
   if (buf) cudaFree(buf);
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
-  // the tuning solves' iteration counts are not the caller's
-  if (rc == BS_OK && cudaMemsetAsync(g->status, 0, kStatusWords * sizeof(int), s) != cudaSuccess)
-    rc = cuda_error(cudaGetLastError(), "coarse_autotune");
   if (rc) return rc;
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);

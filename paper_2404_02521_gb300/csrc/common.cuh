@@ -246,6 +246,9 @@ struct Workspace {
   size_t bytes = 0;
 };
 int ensure(Workspace& w, size_t bytes);
+// The status words around a synchronous solve on stream s (capi.cu).
+int begin_status(bs_grid* g, cudaStream_t s);
+int report_status(bs_grid* g, int bits, cudaStream_t s);
 // Counts a device allocation made by the library (every cudaMalloc / cudaMallocAsync /
 // cudaMallocHost site calls it; read by bs_device_allocations).
 void note_device_alloc();
@@ -260,6 +263,7 @@ struct bs_grid {
   int* status;                 // device int[kStatusWords]: [0] bit 0 = Krylov cap hit, bit 1 =
                                // a cluster exchange timed out; [1] max iterations, [2] total
                                // iterations, [3] solves
+  int failed = 0;              // word [0] as the last synchronous call reported (and cleared) it
   double* dscal;               // device: scalar outputs (defect)
   double* dnorms;              // device: per-slice squared norms / defects
   bsp::Workspace ws_par;       // Parareal F / Gold buffers

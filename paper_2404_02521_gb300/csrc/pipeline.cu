@@ -149,7 +149,7 @@ int parareal_pipelined(bs_grid* g, const bs_params* p, int N, int fine_steps, in
   const bool timing = g_opt.phase_timing != 0;
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> t_fine, t_coarse;
 
-  BS_CUDA_TRY(cudaMemsetAsync(g->status, 0, kStatusWords * sizeof(int), s));
+  if ((rc = begin_status(g, s))) return rc;
   if (!user_u0) {
     if ((rc = launch_payoff(g, dc, u_out, s))) return rc;
     g->n_other += 1;
@@ -271,6 +271,7 @@ int parareal_pipelined(bs_grid* g, const bs_params* p, int N, int fine_steps, in
     if (hstat) {
       *k_done = k + 1;
       BS_CUDA_TRY(cudaStreamSynchronize(sf));
+      if ((rc = report_status(g, hstat, s))) return rc;
       if (hstat & 2)
         return set_error(BS_ERR_CUDA, "parareal_solve: a cluster exchange timed out");
       return set_error(BS_ERR_NOCONV, "parareal_solve: a coarse BiCGSTAB solve hit its iteration cap");
