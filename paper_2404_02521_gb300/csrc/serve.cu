@@ -89,7 +89,7 @@ struct Slot {
   cudaStream_t st = nullptr;
   cudaEvent_t ev = nullptr;
   double* h_defect = nullptr;    // pinned
-  int* h_status = nullptr;       // pinned
+  int* h_status = nullptr;       // pinned: the request's grid's word, its F batch's
   size_t off = 0, bytes = 0;
   float *U = nullptr, *Fb = nullptr, *Gold = nullptr;
   double* norms = nullptr;
@@ -318,8 +318,12 @@ static int launch_group(bs_server* sv, const std::vector<Slot*>& grp) {
   }
   cudaStream_t bst = sv->batch_stream[M];
   bs_grid* cg = sv->class_grid[M];
+  // the batch's own failures (a timed-out exchange), read ahead of the event that its requests wait for
+  BS_CUDA_TRY(cudaMemsetAsync(cg->status, 0, sizeof(int), bst));
   int rc = launch_fine(cg, items.data(), (int)items.size(), fs, bst);
   if (rc) return rc;
+  for (Slot* sl : grp)
+    BS_CUDA_TRY(cudaMemcpyAsync(sl->h_status + 1, cg->status, sizeof(int), cudaMemcpyDeviceToHost, bst));
   sv->launches += fine_launches(cg, items.data(), (int)items.size(), fs);
   sv->fine_batches += 1;
   sv->fine_items += (long long)items.size();
@@ -364,7 +368,7 @@ static int progress(bs_server* sv) {
       sl.phase = PH_READY_F;
     } else if (sl.phase == PH_G) {
       sl.defect = *sl.h_defect;
-      const int st = *sl.h_status;
+      const int st = sl.h_status[0] | sl.h_status[1];
       ++sl.k;
       if (st & 2) {
         sl.result = BS_ERR_CUDA;
@@ -444,7 +448,7 @@ int bs_server_create(const bs_server_config* cfg, bs_server** out) {
     note_device_alloc();
     note_device_alloc();
     if (e == cudaSuccess) e = cudaMallocHost(&sl.h_defect, sizeof(double));
-    if (e == cudaSuccess) e = cudaMallocHost(&sl.h_status, sizeof(int));
+    if (e == cudaSuccess) e = cudaMallocHost(&sl.h_status, 2 * sizeof(int));
   }
   sv->batch_events.resize(64);
   for (auto& be : sv->batch_events)
