@@ -410,14 +410,19 @@ def bs_coarse_variant_info(variant: int, M: int) -> dict:
             "quad": bool(v[4].value)}
 
 
+def bs_grid_status(g: Grid):
+    """(max BiCGSTAB iterations, failure bits -- 1: a solve hit its cap, 2: an exchange timed out --,
+    summed iterations, number of implicit solves) since the last reset, and resets them."""
+    it, fail, tot, ns = C.c_int(0), C.c_int(0), C.c_int(0), C.c_int(0)
+    check(load().bs_grid_stats(g.h, C.byref(it), C.byref(fail), C.byref(tot), C.byref(ns)))
+    return it.value, fail.value, tot.value, ns.value
+
+
 def bs_grid_stats(g: Grid, detail: bool = False):
     """(max BiCGSTAB iterations, any solve hit its cap) since the last reset; with detail,
     also (summed iterations, number of implicit solves)."""
-    it, fail, tot, ns = C.c_int(0), C.c_int(0), C.c_int(0), C.c_int(0)
-    check(load().bs_grid_stats(g.h, C.byref(it), C.byref(fail), C.byref(tot), C.byref(ns)))
-    if detail:
-        return it.value, bool(fail.value), tot.value, ns.value
-    return it.value, bool(fail.value)
+    it, fail, tot, ns = bs_grid_status(g)
+    return (it, bool(fail), tot, ns) if detail else (it, bool(fail))
 
 
 def bs_phase_stats(g: Grid) -> dict:

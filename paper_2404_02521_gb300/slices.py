@@ -11,7 +11,8 @@ eq. (parareal):
      library call -- and sends u_{b_r}^{k+1} to rank r + 1.  A rank whose slices are all
      exact (b_r <= k) neither sweeps nor sends, and its successor does not wait;
   3. the defect of reading c5 from one FP64 max all-reduce of each rank's largest squared
-     norms, delta = sqrt(max ||du||^2) / sqrt(max ||u||^2).
+     norms, delta = sqrt(max ||du||^2) / sqrt(max ||u||^2).  The same reduction carries whether a
+     rank's kernels failed, so that every rank raises after the same iteration.
 
 The all-reduce is started asynchronously and, from the second iteration on while the defect is
 above 10 tol, F of the next iteration is enqueued before its result is known (it only reads
@@ -69,6 +70,11 @@ class SliceBackend:
         """(||U[n]||^2, ||dU[n]||^2) for n in (n_lo, n_hi] (written by the last sweeps)."""
         raise NotImplementedError
 
+    def failure(self) -> int:
+        """Failure bits of the rank's work so far (0: none; 1: a coarse solve hit its iteration
+        cap, 2: an exchange between a kernel's CTAs timed out), once the norms have been read."""
+        return 0
+
     def max_tensor(self, values: Sequence[float]):
         """A float64 tensor of `values` on the device the process group reduces on."""
         raise NotImplementedError
@@ -124,7 +130,7 @@ def parareal_partitioned(backend: SliceBackend, N: int, tol: float, Kmax: int, g
             num2 = max(du for _, du in nrm)
             own_u[lo - a:] = [nu for nu, _ in nrm]   # the rank's slices below lo keep theirs
             den2 = max(own_u)
-        t = backend.max_tensor([num2, den2])
+        t = backend.max_tensor([num2, den2, float(backend.failure())])
         work = dist.all_reduce(t, op=dist.ReduceOp.MAX, group=group, async_op=True)
         work.wait()   # orders the result before later work on the rank's stream
         result = backend.read_async(t)
@@ -137,6 +143,9 @@ def parareal_partitioned(backend: SliceBackend, N: int, tol: float, Kmax: int, g
             backend.fine(max(a, k + 1), b)
             f_done = True
         vals = result()
+        if vals[2]:
+            raise RuntimeError("parareal_partitioned: " + (
+                "an exchange between CTAs timed out" if int(vals[2]) & 2 else "a coarse solve hit its iteration cap"))
         delta = defect_from(vals[0], vals[1])
         defects.append(delta)
         k += 1
@@ -164,6 +173,7 @@ class GpuSlices(SliceBackend):
         self.nrm = torch.zeros(2 * (N + 1), dtype=torch.float64, device=dev)
         self.dev = dev
         self.slice = params.T / N
+        self.krylov = (0, 0, 0)   # of the solves so far: most iterations, all iterations, solves
 
     def initial(self):
         self.lib.bs_payoff(self.g, self.p, self.U[0])
@@ -184,6 +194,11 @@ class GpuSlices(SliceBackend):
     def norms(self, n_lo, n_hi):
         h = self.nrm[2 * (n_lo + 1): 2 * (n_hi + 1)].cpu().tolist()
         return [(h[2 * i], h[2 * i + 1]) for i in range(n_hi - n_lo)]
+
+    def failure(self):
+        iters, bits, total, solves = self.lib.bs_grid_status(self.g)
+        self.krylov = (max(self.krylov[0], iters), self.krylov[1] + total, self.krylov[2] + solves)
+        return bits
 
     def max_tensor(self, values):
         import torch
