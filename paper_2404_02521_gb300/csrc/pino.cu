@@ -56,6 +56,8 @@ struct bs_pino {
   float b2;
   int* err;
   bsp::PinoRes res[2];
+  // the shapes that the cluster path runs (and pino_check accepts)
+  bool clustered() const { return C == 32 && mx == 12 && my == 12 && H % 16 == 0 && H <= 256; }
 };
 
 namespace bsp {
@@ -639,6 +641,49 @@ int pino_error_flag(const bs_pino* net, int* flag) {
   return BS_OK;
 }
 
+// The complex mode matrices w[l][m][c][o] (m = q * mx + kx, n elements in all) as the network paths
+// read them: R in real 2 x 2 blocks, rows (o, re/im), columns (c, re/im); mix, where the cluster path
+// runs the shape, as pino_mix_index lays it out.  Packed here: element by element on the host the two
+// layouts took 12 of the 16 ms of loading a network of four layers.
+__global__ void pino_pack_kernel(const float* __restrict__ re, const float* __restrict__ im, size_t n, int C, int mx,
+                                 int MYx, bf16* __restrict__ R, bf16* __restrict__ mix) {
+  const size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  if (e >= n) return;
+  const int o = (int)(e % C), c = (int)(e / C % C), m = (int)(e / ((size_t)C * C) % MYx);
+  const int l = (int)(e / ((size_t)C * C * MYx));
+  const bf16 wr = __float2bfloat16(re[e]), wi = __float2bfloat16(im[e]);
+  bf16* blk = R + ((size_t)l * MYx + m) * (2 * C) * (2 * C);
+  blk[(2 * o) * (2 * C) + 2 * c] = wr;
+  blk[(2 * o) * (2 * C) + 2 * c + 1] = __float2bfloat16(-im[e]);
+  blk[(2 * o + 1) * (2 * C) + 2 * c] = wi;
+  blk[(2 * o + 1) * (2 * C) + 2 * c + 1] = wr;
+  if (mix) {
+    mix[pino_mix_index(l, m / mx, m % mx, c, o, 0)] = wr;
+    mix[pino_mix_index(l, m / mx, m % mx, c, o, 1)] = wi;
+  }
+}
+
+static int pack_modes(bs_pino* net, const float* spec, size_t n) {   // spec: host, re[n] then im[n]
+  float* raw = nullptr;
+  int rc = dev_alloc((void**)&raw, 2 * n * sizeof(float));
+  if (rc) return rc;
+  if ((rc = dev_alloc((void**)&net->R, 4 * n * sizeof(bf16))) == BS_OK && net->clustered())
+    rc = dev_alloc((void**)&net->mix, 2 * n * sizeof(bf16));
+  cudaError_t e = cudaSuccess;
+  if (!rc) {
+    e = cudaMemcpy(raw, spec, 2 * n * sizeof(float), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+      pino_pack_kernel<<<(unsigned)((n + 255) / 256), 256>>>(raw, raw + n, n, net->C, net->mx, 2 * net->my * net->mx,
+                                                             net->R, net->mix);
+      e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);   // the network may be used on any stream
+    if (e != cudaSuccess) rc = cuda_error(e, "pino_load");
+  }
+  cudaFree(raw);
+  return rc;
+}
+
 }  // namespace bsp
 
 using namespace bsp;
@@ -670,27 +715,14 @@ extern "C" int pino_load(const char* path, bs_pino** out) {
   const float* fp = reinterpret_cast<const float*>(buf.data() + 40);
   auto take = [&](size_t n) { std::vector<float> v(fp, fp + n); fp += n; return v; };
   std::vector<float> lift_w = take((size_t)cin * C), lift_b = take(C);
-  std::vector<float> sre = take((size_t)L * MYx * C * C), sim = take((size_t)L * MYx * C * C);
+  const size_t nspec = (size_t)L * MYx * C * C;
+  const float* spec = fp;   // re, im
+  fp += 2 * nspec;
   std::vector<float> pw_w = take((size_t)L * C * C), pw_b = take((size_t)L * C);
   std::vector<float> p1w = take((size_t)C * H), p1b = take(H), p2w = take(H), p2b = take(1);
 
   bs_pino* net = new bs_pino();
-  std::memset(net, 0, sizeof(*net));
   net->cin = cin; net->C = C; net->mx = mx; net->my = my; net->L = L; net->H = H; net->b2 = p2b[0];
-  // complex mode matrices in real 2x2 block form: rows (o, re/im), columns (c, re/im)
-  std::vector<bf16> R((size_t)L * MYx * 2 * C * 2 * C);
-  for (int l = 0; l < L; ++l)
-    for (size_t m = 0; m < MYx; ++m)
-      for (int c = 0; c < C; ++c)
-        for (int o = 0; o < C; ++o) {
-          const size_t src = (((size_t)l * MYx + m) * C + c) * C + o;
-          const float re = sre[src], im = sim[src];
-          bf16* blk = R.data() + ((size_t)l * MYx + m) * (2 * C) * (2 * C);
-          blk[(2 * o) * (2 * C) + 2 * c] = __float2bfloat16(re);
-          blk[(2 * o) * (2 * C) + 2 * c + 1] = __float2bfloat16(-im);
-          blk[(2 * o + 1) * (2 * C) + 2 * c] = __float2bfloat16(im);
-          blk[(2 * o + 1) * (2 * C) + 2 * c + 1] = __float2bfloat16(re);
-        }
   std::vector<bf16> Wpw((size_t)L * C * C), W1((size_t)H * C);
   for (int l = 0; l < L; ++l)
     for (int c = 0; c < C; ++c)
@@ -698,22 +730,14 @@ extern "C" int pino_load(const char* path, bs_pino** out) {
   for (int c = 0; c < C; ++c)
     for (int h = 0; h < H; ++h) W1[(size_t)h * C + c] = __float2bfloat16(p1w[(size_t)c * H + h]);
   int rc;
-  if (C == 32 && mx == 12 && my == 12 && H % 16 == 0 && H <= 256) {
-    std::vector<bf16> mix((size_t)L * MYx * 2 * C * C), wc;
+  if (net->clustered()) {
+    std::vector<bf16> wc;
     for (int l = 0; l < L; ++l) {
-      for (size_t m = 0; m < MYx; ++m)
-        for (int c = 0; c < C; ++c)
-          for (int o = 0; o < C; ++o) {
-            const size_t src = (((size_t)l * MYx + m) * C + c) * C + o;
-            mix[pino_mix_index(l, (int)m / mx, (int)m % mx, c, o, 0)] = __float2bfloat16(sre[src]);
-            mix[pino_mix_index(l, (int)m / mx, (int)m % mx, c, o, 1)] = __float2bfloat16(sim[src]);
-          }
       const auto w = Wpw.begin() + (long)l * C * C;
       const std::vector<bf16> one = canonical(std::vector<bf16>(w, w + C * C), C, C);
       wc.insert(wc.end(), one.begin(), one.end());
     }
-    if ((rc = upload(&net->mix, mix)) || (rc = upload(&net->Wpw_c, wc)) ||
-        (rc = upload(&net->W1_c, canonical(W1, H, C)))) {
+    if ((rc = upload(&net->Wpw_c, wc)) || (rc = upload(&net->W1_c, canonical(W1, H, C)))) {
       pino_destroy(net);
       return rc;
     }
@@ -723,7 +747,7 @@ extern "C" int pino_load(const char* path, bs_pino** out) {
   p1b.resize(Hp, 0.f);
   p2w.resize(Hp, 0.f);
   if ((rc = upload(&net->lift_w, lift_w)) || (rc = upload(&net->lift_b, lift_b)) ||
-      (rc = upload(&net->R, R)) || (rc = upload(&net->Wpw, Wpw)) || (rc = upload(&net->pw_b, pw_b)) ||
+      (rc = pack_modes(net, spec, nspec)) || (rc = upload(&net->Wpw, Wpw)) || (rc = upload(&net->pw_b, pw_b)) ||
       (rc = upload(&net->W1, W1)) || (rc = upload(&net->b1, p1b)) || (rc = upload(&net->w2, p2w)) ||
       (rc = dev_alloc((void**)&net->err, sizeof(int)))) {
     pino_destroy(net);

@@ -52,7 +52,7 @@ struct PinoClusterNet {
 
 // Element (c -> o, re/im) of layer l's matrix of mode (q, kx) in PinoClusterNet::mix.  A unit is
 // four consecutive q at one kx; a lane holds four outputs and four inputs of a half unit.
-inline size_t pino_mix_index(int l, int q, int kx, int c, int o, int ri) {
+__host__ __device__ inline size_t pino_mix_index(int l, int q, int kx, int c, int o, int ri) {
   const int unit = (q >> 2) * 12 + kx, lane = (c >> 2) * 4 + ((o & 15) >> 2);
   return ((((((size_t)l * 72 + unit) * 2 + (o >> 4)) * 4 + (q & 3)) * 4 + (c & 3)) * 32 + lane) * 8 +
          (size_t)(o & 3) * 2 + ri;
