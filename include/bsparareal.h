@@ -141,7 +141,7 @@ int bs_payoff3(int M, double xmax, const bs_params3* p, float* u, bs_stream stre
  * float[M^3] (may alias).  Allocates its workspace stream-ordered (6 M^3 floats per state).
  * The first step starts from a zero increment (solved to q^m <= 2^-22), the second from the
  * previous one (2^-10), later ones from the extrapolation of the previous two (step n to
- * min(n / 128, 0.5), an even count above 1/4).
+ * min(n^2 / 2048, n / 192, 0.5), an even count above 1/4, and to 1/3 where drift exceeds diffusion).
  * Asynchronous.  Results for a state do not depend on B or on the other states.
  * Errors: BS_ERR_ARG (as bs_payoff3; NULL pointers, B < 1, dtau <= 0, q >= 0.8),
  * BS_ERR_CUDA. */

@@ -8,7 +8,7 @@
 // second from the previous increment, later ones from the extrapolation of the previous two.  u is
 // carried as a compensated (hi, lo) FP32 pair.  Starting every step from the previous
 // increment took 22 sweeps per step at q = 0.72 (64^3, dtau = 1/640) where the extrapolation
-// takes 13 falling to 4: 16 states, 40 steps, 24.4 -> 9.7 ms, with the same error against 64
+// takes 19 falling to 5: 16 states, 40 steps, 24.0 -> 11.0 ms, with the same error against 64
 // bits (1.6e-6; 3.6e-6 and 2.2e-6 on longer runs, all unchanged to three digits).
 // Stencil coefficients are products of host-rounded FP32 constants and exact integer node
 // indices (x_p = i_p h, so h cancels).
@@ -21,8 +21,7 @@
 // column (i, j) up through the block's planes.  The first sweep of a step also stages hi and
 // forms b = dtau R_h hi (the RHS phase); the last sweep also adds the increment to (hi, lo)
 // (APPLY) and writes the far faces of the next step (FACE).  So a step is its sweeps alone;
-// f3_phase_kernel remains only for the INIT and OUT passes of a launch (and the FACE pass
-// before the first step).
+// f3_phase_kernel remains only for the passes before the first step (INIT) and after the last (OUT).
 //
 // Layout: u[(k*M + j)*M + i] with i the index of asset 1 (fastest), j of asset 2, k of
 // asset 3.  Nodes with an index M - 1 carry Dirichlet data; nodes with an index 0 carry the
@@ -244,9 +243,12 @@ double f3_contraction(int M, const bs_params3& p, double dtau) {
 // Sweeps of step `step` of a propagation, by how its solve starts: from zero, from the
 // previous increment, or from the extrapolation of the previous two.  An extrapolated start is
 // off by a mode's second difference in time, and the modes that have survived n steps decay by
-// about 1/n per step, so the reduction that the solve owes falls with n.  A fixed 2^-6 up to
-// step 16 and 1/2 from there takes a tenth fewer sweeps, but on a white-noise state left 6e-6
-// (24^3, q = 0.72, 40 steps) where this leaves the FP32 rounding's 1e-6.  A target above 1/4
+// about 1/n per step, so the reduction that the solve owes falls with n, at first with n^2.  On
+// white-noise states of 17^3 to 64^3, 4 to 80 steps at q = 0.72, the error is within 3.5% of the
+// one with every step from the previous increment to 2^-10 (1.26e-7 after 4 steps at 17^3, 9.8e-7
+// after 40 at 24^3, 1.80e-6 at 48^3; on payoffs the same to three digits).  n / 128 without the
+// quadratic start takes a tenth fewer sweeps and left 2.8e-7 after those 4 steps; a fixed 2^-6 up to
+// step 16 and 1/2 from there a fifth fewer, and 6e-6 after 40 at 24^3.  A target above 1/4
 // takes an even count: the error recurrence e_{t+1} = l^m (2 e_t - e_{t-1}) of an extrapolated
 // start has a root beyond 1 where l^m < -1/3 (l an eigenvalue of the sweep, which can be
 // negative).
@@ -256,7 +258,7 @@ constexpr int kF3ExtrapStart = 2;
 static int f3_sweeps(double q, double skew, int step) {
   const double target = step == 0               ? 1.0 / 4194304.0
                         : step < kF3ExtrapStart ? 1.0 / 1024.0
-                                                : std::fmin(step / 128.0, 0.5);
+                                                : std::fmin(std::fmin(step * step / 2048.0, step / 192.0), 0.5);
   if (q <= 0.0) return 2;
   const int m = std::max(2, (int)std::ceil(std::log(target) / std::log(q)));
   return step < kF3ExtrapStart ? m : extrap_sweeps(q, skew, target > 0.25 ? (m + 1) & ~1 : m);
