@@ -237,15 +237,6 @@ __device__ __forceinline__ void xround(Xchg& xs, const float (&v)[NV], float (&t
   ++xs.round;
 }
 
-// The quotients of the Krylov scalars, on the serial path of every iteration: 2 ulp and no
-// correction steps.  They need not be rounded: r, s and x follow whatever alpha and omega they are
-// given, and beta only sets the next direction.  (A divisor that is subnormal or beyond 2^126 keeps the
-// rounded quotient: its reciprocal is out of range.)
-__device__ __forceinline__ float krylov_div(float a, float b) {
-  const float m = fabsf(b);
-  return m > 1.2e-38f && m < 8.0e37f ? __fdividef(a, b) : a / b;
-}
-
 // v with its sign flipped where bit k of `bits` is set: the product with the shadow residual
 // r^ = sign(r_0) of row k.
 __device__ __forceinline__ float signed_by(float v, uint32_t bits, int k) {
@@ -687,7 +678,7 @@ __global__ void __launch_bounds__(CFG::NT, 1) sweep_band_kernel(const __grid_con
             if (xs.dead) { conv = true; break; }
             if (ta[1] <= stop2) { conv = true; break; }
             if (ta[0] == 0.f) { fail = true; break; }
-            const float af = krylov_div(rho, ta[0]);
+            const float af = rho / ta[0];
             // s = r - alpha v (rr holds s from here on), own rows and halo rows
 #pragma unroll
             for (int k = 0; k < K; ++k) {
@@ -742,11 +733,11 @@ __global__ void __launch_bounds__(CFG::NT, 1) sweep_band_kernel(const __grid_con
             float tb[4];
             xround<CFG, 4>(xs, p2, tb, rank, C, halo_bytes);
             if (xs.dead) { conv = true; break; }
-            const float of = tb[1] > 0.f ? krylov_div(tb[0], tb[1]) : 0.f;
+            const float of = tb[1] > 0.f ? tb[0] / tb[1] : 0.f;
             const float rho_new = tb[2] - of * tb[3];
             float bf = 0.f;
             if (of == 0.f || rho == 0.f) fail = true;
-            else bf = krylov_div(rho_new, rho) * krylov_div(af, of);
+            else bf = (rho_new / rho) * (af / of);
             rho = rho_new;
             // x += omega s (POLY: omega M^{-1} s) ;  r = s - omega t ;  p = r + beta (p - omega v)
 #pragma unroll
