@@ -535,9 +535,9 @@ pino_cluster_kernel(const __grid_constant__ PinoClusterNet net, const __grid_con
       // K = 24 .. 31: the bias in three parts, exactly, against ones in the inverse x-DFT
       if (tid < ROWS * 32) {
         const float bias = net.pw_b[l * 32 + lane];
-        const float hi = bf_lo(pack_bf16(bias, 0.f));
-        const bool fin = fabsf(hi) < INFINITY;
-        const float mid = fin ? bf_lo(pack_bf16(bias - hi, 0.f)) : 0.f, lo = fin ? (bias - hi) - mid : 0.f;
+        // eight leading bits each, cut off: rounded, the largest finite values would become infinite
+        const float hi = fabsf(bias) < INFINITY ? bf_hi(__float_as_uint(bias)) : bias;
+        const float mid = hi == bias ? 0.f : bf_hi(__float_as_uint(bias - hi)), lo = hi == bias ? 0.f : (bias - hi) - mid;
         *reinterpret_cast<uint4*>(smem + F::YZ + (tid >> 5) * 2048 + (lane >> 3) * 512 + 384 + (lane & 7) * 16) =
             make_uint4(pack_bf16(hi, mid), pack_bf16(lo, 0.f), 0, 0);
       }
