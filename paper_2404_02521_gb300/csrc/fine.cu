@@ -88,11 +88,12 @@ static FineLayout make_layout(int M, int tc, int tr, int C, int hmin) {
 // Estimated time of a late (two-sweep) step of nb states, in SM clocks: waves of clusters times
 // the clocks of a CTA's step (fitted to 2.4k to 6.5k clocks measured for 1024 to 8192 nodes per
 // CTA) and, over several regions, a launch's load, setup and store (about 27k clocks at 8192
-// nodes) per step.
+// nodes) per step.  A layout without a known capacity (clusters above 8 CTAs may not fit the device)
+// comes after every layout with one.
 static double layout_cost(const FineLayout& y, int nb) {
   const int cap = layout_capacity(y);
   const double clusters = (double)nb * y.ntx * y.nty;
-  const double waves = cap > 0 ? std::ceil(clusters / cap) : clusters * y.C / 100.0;
+  const double waves = cap > 0 ? std::ceil(clusters / cap) : 1e9 * clusters * y.C;
   const double nodes = 32.0 * y.tc * kFineWarps * y.tr;
   double t = 1800.0 + 0.57 * nodes;
   if (y.ntx * y.nty > 1) t += (3000.0 + 1.3 * nodes) / std::max(1, std::min(y.H, 1 << 10) / 2);

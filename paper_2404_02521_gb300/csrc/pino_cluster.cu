@@ -29,6 +29,9 @@
 // share one region, the y-DFT and the x-DFT matrices another; the order is given at each).
 // Every wait is bounded; a CTA whose wait ran out records the error, stops waiting and still
 // takes part in the barriers.
+#include <map>
+#include <mutex>
+
 #include "cluster_async.cuh"
 #include "pino.cuh"
 
@@ -690,17 +693,30 @@ void pc_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int B, cudaSt
   cfg.numAttrs = 1;
 }
 
-// clusters that run at once (0 if the size cannot be launched)
+// clusters that the current device runs at once (0 if the size cannot be launched), measured once per
+// device
 template <int CL>
 int pc_capacity() {
-  static const int n = [] {
-    int v = 0;
-    if (pc_attributes<CL>() != cudaSuccess) return 0;
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute attr[1];
-    pc_config<CL>(cfg, attr, 1, nullptr);
-    return cudaOccupancyMaxActiveClusters(&v, pino_cluster_kernel<CL>, &cfg) == cudaSuccess ? v : 0;
-  }();
+  static std::mutex mu;
+  static std::map<int, int> cache;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  std::lock_guard<std::mutex> lock(mu);
+  const auto it = cache.find(dev);
+  if (it != cache.end()) return it->second;
+  int n = 0;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[1];
+  pc_config<CL>(cfg, attr, 1, nullptr);
+  if (pc_attributes<CL>() != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, pino_cluster_kernel<CL>, &cfg) != cudaSuccess) {
+    cudaGetLastError();   // a size that cannot be launched is not the next call's error
+    n = 0;
+  }
+  cache[dev] = n;
   return n;
 }
 
