@@ -207,12 +207,12 @@ def barrier(world):
         dist.barrier()
 
 
-FINE_SOURCES = ["paper_2404_02521_gb300/csrc/" + f for f in ("fine.cu", "fine_tile.cuh", "fine_launch.cuh", "common.cuh")]
-KERNEL_SOURCES = {
-    "fine_tile_kernel": FINE_SOURCES,
-    "sweep_band_kernel": ["paper_2404_02521_gb300/csrc/coarse.cu", "paper_2404_02521_gb300/csrc/band.cuh",
-                          "paper_2404_02521_gb300/csrc/common.cuh"],
-}
+# what a kernel is compiled from: its files and every header of theirs
+KERNEL_SOURCES = {k: ["paper_2404_02521_gb300/csrc/" + f for f in v] for k, v in {
+    "fine_tile_kernel": ("fine.cu", "fine_wa.cu", "fine_wb.cu", "fine_wc.cu", "fine_wd.cu", "fine_we.cu", "fine_tile.cuh",
+                         "fine_launch.cuh", "band.cuh", "cluster_async.cuh", "common.cuh"),
+    "sweep_band_kernel": ("coarse.cu", "band.cuh", "cluster_async.cuh", "common.cuh"),
+}.items()}
 
 
 def traffic_entry(kernel):
