@@ -20,10 +20,6 @@ __device__ __forceinline__ uint32_t cluster_addr(uint32_t local, int rank) {
 __device__ __forceinline__ void mbar_init(uint64_t* mb, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_addr(mb)), "r"(count) : "memory");
 }
-// one arrival on an mbarrier of this CTA
-__device__ __forceinline__ void mbar_arrive(uint64_t* mb) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_addr(mb)) : "memory");
-}
 // one arrival that announces the bytes the phase's asynchronous stores will complete
 __device__ __forceinline__ void mbar_arm(uint64_t* mb, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_addr(mb)), "r"(bytes)
