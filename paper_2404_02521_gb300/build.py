@@ -21,11 +21,14 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # host code: no contraction into fused multiply-adds, so x86 and Arm hosts round alike
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off",
          "--expt-relaxed-constexpr"]
-# the fine stepper's device code, too: its layouts and launch plans instantiate the same
-# stencil in different kernels, and only without implicit contraction do they round alike
-# (its multiply-adds are written as explicit fused operations)
-FILE_FLAGS = {f: ["-fmad=false"] for f in ("fine.cu", "fine_wa.cu", "fine_wb.cu", "fine_wc.cu", "fine_wd.cu",
-                                           "fine_we.cu")}
+# the device code of the fine stepper and of the grid solver, too: their layouts and launch plans
+# instantiate the same stencil in different kernels, and only without implicit contraction do they
+# round alike (their multiply-adds are written as explicit fused operations)
+EXACT = ("fine.cu", "fine_w", "coarse_grid.cu")
+
+
+def file_flags(name: str):
+    return ["-fmad=false"] if name.startswith(EXACT) else []
 
 
 def nvcc() -> str:
@@ -65,7 +68,7 @@ def build(force: bool = False, verbose: bool = False, extra=()) -> str:
 
     def compile_one(src):
         obj = os.path.join(BUILD, os.path.basename(src).replace(".cu", ".o"))
-        cmd = [cc, *ARCH, *FLAGS, *FILE_FLAGS.get(os.path.basename(src), []), *extra, "-I", INCLUDE, "-c", src,
+        cmd = [cc, *ARCH, *FLAGS, *file_flags(os.path.basename(src)), *extra, "-I", INCLUDE, "-c", src,
                "-o", obj]
         if verbose:
             print(" ".join(cmd), flush=True)

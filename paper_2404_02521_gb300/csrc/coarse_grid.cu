@@ -49,10 +49,25 @@ struct CgArgs {
   float h;
 };
 
-// weighted neighbours of the entry y of a staged operand
-__device__ __forceinline__ float cg_off(const float* y, float ce, float cw, float cs, float cn, float cg) {
-  return ce * y[1] + cw * y[-1] + cs * y[kCgS] + cn * y[-kCgS] +
-         cg * ((y[kCgS + 1] - y[-kCgS + 1]) - (y[kCgS - 1] - y[-kCgS - 1]));
+// Every multiply-add of this file is explicit and it is compiled without implicit contraction, so a ring
+// node of M^{-1} p equals its owner's bit for bit.
+
+// row_coefs with the drift fused in
+__device__ __forceinline__ void cg_row(const ItemDesc& d, int j, float& cs, float& cn, float& gj) {
+  gj = (float)j;
+  const float b = d.ay * (gj * gj);
+  cs = fmaf(d.my, gj, b);
+  cn = fmaf(-d.my, gj, b);
+}
+
+// weighted neighbours of a node
+__device__ __forceinline__ float cg_off(float nW, float nC, float nE, float cW, float cE, float sW, float sC, float sE,
+                                        float ce, float cw, float cs, float cn, float cg) {
+  float t = ce * cE;
+  t = fmaf(cw, cW, t);
+  t = fmaf(cs, sC, t);
+  t = fmaf(cn, nC, t);
+  return fmaf(cg, (sE - nE) - (sW - nW), t);
 }
 
 // ONE: every block owns one tile, whose Krylov vectors stay in registers; only the nodes that a
@@ -159,9 +174,8 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
     for (int k = 0; k < K; ++k) {
       const float sW = y[(k + 1) * kCgS - 1], sC = y[(k + 1) * kCgS], sE = y[(k + 1) * kCgS + 1];
       float cs, cn, gj;
-      row_coefs(d, j0 + r0 + k, cs, cn, gj);
-      const float off = ce * cE + cw * cW + cs * sC + cn * nC + cgi * gj * ((sE - nE) - (sW - nW));
-      f(k, cC, cC - id[k] * off);
+      cg_row(d, j0 + r0 + k, cs, cn, gj);
+      f(k, cC, fmaf(-id[k], cg_off(nW, nC, nE, cW, cE, sW, sC, sE, ce, cw, cs, cn, cgi * gj), cC));
       nW = cW; nC = cC; nE = cE;
       cW = sW; cC = sC; cE = sE;
     }
@@ -188,9 +202,12 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
       if (i >= 0 && i < M - 1 && j >= 0 && j < M - 1) {
         float e, w, g, cs, cn, gj;
         column_coefs(d, i, e, w, g);
-        row_coefs(d, j, cs, cn, gj);
+        cg_row(d, j, cs, cn, gj);
         const float* y = P + row * kCgS + c;
-        val = fmaf(2.f, y[0], -(y[0] - inv_diag(d, i, j) * cg_off(y, e, w, cs, cn, g * gj)));
+        val = fmaf(2.f, y[0], -fmaf(-inv_diag(d, i, j),
+                                    cg_off(y[-kCgS - 1], y[-kCgS], y[-kCgS + 1], y[-1], y[1], y[kCgS - 1], y[kCgS],
+                                           y[kCgS + 1], e, w, cs, cn, g * gj),
+                                    y[0]));
       }
       Q[row * kCgS + c] = val;
     }
@@ -232,8 +249,8 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
             const int i = i0 + tc, j = j0 + r0 + k;
             if (i == M - 1 || j == M - 1) gu[e] = far_field(pf, i * ca.h, j * ca.h, tau_new);
             const float d1 = gx[e], d2 = gxp[e];
-            if (nhist >= 3) gx[e] = 3.f * (d1 - d2) + gxq[e];
-            else if (nhist == 2) gx[e] = 2.f * d1 - d2;
+            if (nhist >= 3) gx[e] = fmaf(3.f, d1 - d2, gxq[e]);
+            else if (nhist == 2) gx[e] = fmaf(2.f, d1, -d2);
             gxq[e] = d2;
             gxp[e] = d1;
           });
@@ -259,10 +276,14 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
 #pragma unroll
             for (int k = 0; k < K; ++k, y += kCgS) {
               float cs, cn, gj;
-              row_coefs(d, j0 + r0 + k, cs, cn, gj);
+              cg_row(d, j0 + r0 + k, cs, cn, gj);
               const float c = y[0];
-              const float b = ce * (y[1] - c) - cw * (c - y[-1]) + cs * (y[kCgS] - c) - cn * (c - y[-kCgS]) +
-                              cgi * gj * ((y[kCgS + 1] - y[-kCgS + 1]) - (y[kCgS - 1] - y[-kCgS - 1])) - rdt * c;
+              float b = ce * (y[1] - c);
+              b = fmaf(-cw, c - y[-1], b);
+              b = fmaf(cs, y[kCgS] - c, b);
+              b = fmaf(-cn, c - y[-kCgS], b);
+              b = fmaf(cgi * gj, (y[kCgS + 1] - y[-kCgS + 1]) - (y[kCgS - 1] - y[-kCgS - 1]), b);
+              b = fmaf(-rdt, c, b);
               const float bh = b * id[k];
               r[k] = rh[k] = p[k] = bh - ax[k];
               sums[0] = fmaf(bh, bh, sums[0]);
@@ -372,7 +393,7 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
             grid.sum(sb);
             open = true;
             omega = sb[1] > 0.f ? sb[0] / sb[1] : 0.f;
-            const float rho_new = sb[2] - omega * sb[3];
+            const float rho_new = fmaf(-omega, sb[3], sb[2]);
             if (omega == 0.f || rho == 0.f) {
               fail = true;
               beta = 0.f;

@@ -1,4 +1,5 @@
-"""The files behind a kernel decide whether a committed capture is still the kernel's."""
+"""The files behind a kernel decide whether a committed capture is still the kernel's, and whether its layouts
+round alike."""
 import os
 import re
 
@@ -29,3 +30,14 @@ def test_captures_follow_every_source(kernel):
     if kernel == "fine_tile_kernel":
         home |= {f for f, t in text.items() if "BS_FINE_INSTANCE(" in t} | {"fine.cu"}
     assert listed == closure(home)
+
+
+def test_layouts_that_agree_bitwise_are_compiled_without_contraction():
+    # F's planner and every file that instantiates its tiles, and the grid solver's layouts
+    exact = [f for f in os.listdir(build.CSRC) if f.endswith(".cu") and
+             ("BS_FINE_INSTANCE(" in open(os.path.join(build.CSRC, f)).read() or f in ("fine.cu", "coarse_grid.cu"))]
+    assert len(exact) > 2
+    for f in exact + ["fine_wz.cu"]:
+        assert "-fmad=false" in build.file_flags(f), f
+    for f in ("coarse.cu", "fine3.cu", "pino.cu"):
+        assert build.file_flags(f) == [], f
