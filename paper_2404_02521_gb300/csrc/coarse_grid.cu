@@ -3,9 +3,11 @@
 // preconditioned with M^{-1} = 2I - A^, extrapolated first guesses) with its vectors in a global
 // workspace, one cooperative launch per call.
 //
-// A state is owned by a group of blocks, one tile of kCgW x kCgH nodes per block where the GPU
-// holds that many blocks, else several.  An iteration is two passes over the group's tiles, each
-// followed by one barrier of the group that also carries its dot products:
+// A state is owned by a group of blocks, one tile of kCgW x kCgH nodes per block or several (cg_layout).
+// Where a state may get more or fewer blocks, its sums are kept per tile and added in the tiles'
+// order; every rounding is explicit, so its result does not depend on how many it got.  An iteration
+// is two passes over the group's tiles, each followed by one barrier of the group that also carries
+// its dot products:
 //   A  x += omega M^{-1} s, r = s - omega t, p = r + beta (p - omega v), v = A^ M^{-1} p:
 //      (r^, v), (r, r)
 //   B  x += alpha M^{-1} p, s = r - alpha v, t = A^ M^{-1} s: (t, s), (t, t), (r^, s), (r^, t)
@@ -18,10 +20,10 @@
 // iteration, 10.6 us at 512 x 512 on 128 blocks (49.5 us in the former layout, one cluster of 16
 // SMs with eight cluster barriers and every vector update through L2).  64 x 32 tiles keep a
 // 512 x 512 state's vectors in the registers of one block per tile (12% of the staged nodes
-// are halo); up to 304 tiles are resident, above that (about 780 x 780) a block passes its
-// tiles through the workspace (1024 x 1024: 29.5 us per iteration, 172 before).  States of a batched
-// launch run side by side in as many groups of blocks as the GPU holds, then one after
-// another (10 states of 301 x 301: 2.5 us per iteration, 7.0 before).
+// are halo); up to 304 tiles are resident, above that (about 770 x 770) a block passes its
+// tiles through the workspace (1024 x 1024: 25.4 us per iteration, 172 on one cluster).  States of a
+// batched launch run side by side in groups of blocks, then one after another (10 states of
+// 301 x 301: 2.5 us per iteration and state, 7.0 on clusters).
 #include <algorithm>
 #include <mutex>
 
@@ -38,19 +40,22 @@ constexpr int kCgHalo = 2 * 2 * kCgS + 2 * 2 * kCgH;          // nodes of an ope
 constexpr int kCgRing = 2 * (kCgW + 2) + 2 * kCgH;            // nodes of its inner ring
 constexpr int kCgAttempts = 3;                      // BiCGSTAB starts per implicit step
 constexpr int kCgVectors = 13;
+constexpr int kCgArrivalStride = 32;                // a cache line per group's counter
 
 struct CgArgs {
   ItemDesc d;        // dtau = coarse step
   SweepArgs a;
   float* ws;         // per group: kCgVectors vectors of M*M
-  GridWords* words;  // per group, zero at launch
-  double2* npart;    // per group: [2][kGridMaxBlocks] (norms)
-  int M, group_blocks, groups;
+  float4* partials;  // per group: [2][tiles], the tiles' sums
+  double2* npart;    // [2][group_blocks]: norms of a sweep (one group)
+  unsigned* arrivals;   // per group, kCgArrivalStride apart, zero at launch
+  int M, tiles, group_blocks, groups;
   float h;
 };
 
-// Every multiply-add of this file is explicit and it is compiled without implicit contraction, so a ring
-// node of M^{-1} p equals its owner's bit for bit.
+// Every multiply-add of this file is explicit and it is compiled without implicit contraction: a ring
+// node of M^{-1} p equals its owner's bit for bit, and a state's result is the same whether its tiles
+// stay in registers or not.
 
 // row_coefs with the drift fused in
 __device__ __forceinline__ void cg_row(const ItemDesc& d, int j, float& cs, float& cn, float& gj) {
@@ -72,16 +77,18 @@ __device__ __forceinline__ float cg_off(float nW, float nC, float nE, float cW, 
 
 // ONE: every block owns one tile, whose Krylov vectors stay in registers; only the nodes that a
 // neighbour stages (two rows and columns along the tile's edges) are written to the workspace.
-// Otherwise a pass loads and stores them tile by tile.
-template <bool ONE>
-__global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(const __grid_constant__ CgArgs ca) {
+// Otherwise a pass loads and stores them tile by tile.  PER_SM: blocks that share an SM.  A block that
+// has an SM to itself adds the sums of its tiles in registers, others keep them per tile (TILE_SUMS).
+template <bool ONE, int PER_SM>
+__global__ void __launch_bounds__(kCgThreads, PER_SM) sweep_grid_kernel(const __grid_constant__ CgArgs ca) {
   constexpr int K = kCgK;
+  constexpr bool TILE_SUMS = PER_SM > 1;
   const ItemDesc& d = ca.d;
   const SweepArgs& a = ca.a;
   const int M = ca.M, tid = threadIdx.x;
   const size_t MM = (size_t)M * M;
   const int group = blockIdx.x / ca.group_blocks;
-  GridGroup<kCgThreads> grid{ca.words + group, a.status,
+  GridGroup<kCgThreads> grid{ca.arrivals + group * kCgArrivalStride, ca.partials + (size_t)group * 2 * ca.tiles, ca.tiles, a.status,
                              (int)blockIdx.x % ca.group_blocks, ca.group_blocks, tid};
   float* w0 = ca.ws + (size_t)group * kCgVectors * MM;
   float *const gu = w0, *const gx = w0 + MM, *const gxp = w0 + 2 * MM, *const gxq = w0 + 3 * MM, *const gr = w0 + 4 * MM,
@@ -91,7 +98,7 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
   __shared__ float P[kCgS * (kCgH + 4)], Q[kCgS * (kCgH + 4)];
   const PayoffF pf = make_payoff(d);
   const float rdt = d.rdt, tol = (float)a.tol;
-  const int tiles_i = (M + kCgW - 1) / kCgW, tiles = tiles_i * ((M + kCgH - 1) / kCgH);
+  const int tiles_i = (M + kCgW - 1) / kCgW, tiles = ca.tiles;
   const int tc = tid % kCgW, r0 = tid / kCgW * K;   // the thread's column and first row of a tile
   const int L0 = (r0 + 2) * kCgS + tc + 2;          // and its index in P and Q
   int i0 = 0, j0 = 0;
@@ -110,14 +117,19 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
   };
   auto each_tile = [&](auto&& body) {
     if constexpr (ONE) {
-      body();
+      body(grid.block);
     } else {
       for (int tile = grid.block; tile < tiles; tile += grid.blocks) {
         enter(tile);
-        body();
+        body(tile);
         __syncthreads();   // the staged operands are rewritten
+        if (TILE_SUMS) grid.flush();
       }
     }
+  };
+  auto reduce4 = [&](float (&v)[4]) {
+    if (TILE_SUMS) grid.total(v, tiles);
+    else grid.sum(v);
   };
   if constexpr (ONE) enter(grid.block);
   // f(k, e) for the nodes of the strip that lie in the grid, e their index
@@ -140,6 +152,10 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
     strip([&](int k, size_t e) {
       if (!ONE || tc < 2 || tc >= kCgW - 2 || r0 + k < 2 || r0 + k >= kCgH - 2) g[e] = v[k];
     });
+  };
+  auto advance = [](float (&y)[K], float a, const float (&d)[K]) {   // y += a d
+#pragma unroll
+    for (int k = 0; k < K; ++k) y[k] = fmaf(a, d[k], y[k]);
   };
   // own nodes of an operand into its tile
   auto put = [&](float* dst, const float (&v)[K]) {
@@ -223,6 +239,13 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
   bool failed = false;
   // the strip's x, r (s after an iteration's first pass), r^, p, v, t and M^{-1} p (then M^{-1} s)
   float x[K], r[K], rh[K], p[K], v[K], t[K], q[K];
+  // of a tile in the workspace: where a block has its SM's registers, its loads are all in flight at once
+  // and its stores come last; else x is done with before the others are loaded
+  constexpr bool EARLY = PER_SM == 1;
+  auto advance_x = [&](float a) {
+    advance(x, a, q);
+    store(gx, x);
+  };
 
   for (int st = group; st < nstates && !grid.dead; st += ca.groups) {
     const PropItem pit = batched ? a.prop[st] : PropItem{a.in, a.out, d.tau0};
@@ -230,7 +253,7 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
                        : a.mode == SWEEP_INIT ? a.U + (size_t)n_lo * MM
                        : n_lo == a.n_first    ? a.Gold + (size_t)a.n_first * MM   // G(u_k) unchanged: G_old_k
                                               : a.U + (size_t)n_lo * MM;
-    each_tile([&] {
+    each_tile([&](int) {
       strip([&](int, size_t e) {
         gu[e] = src[e];
         gx[e] = 0.f;
@@ -244,7 +267,7 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
       for (int cstep = 0; cstep < (skip_g ? 0 : a.csteps) && !grid.dead; ++cstep) {
         const float tau_new = (float)(pit.tau0 + a.slice_len * n + (cstep + 1) * d.dtau);
         // far-field data, and the first guess 3 d_{m-1} - 3 d_{m-2} + d_{m-3} (gx holds d_{m-1})
-        each_tile([&] {
+        each_tile([&](int) {
           strip([&](int k, size_t e) {
             const int i = i0 + tc, j = j0 + r0 + k;
             if (i == M - 1 || j == M - 1) gu[e] = far_field(pf, i * ca.h, j * ca.h, tau_new);
@@ -262,7 +285,8 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
           grid.barrier();   // the owners' u and x are visible
           // b^ = D^{-1} dtau R_h u;  r = r^ = p = b^ - A^ x
           float sums[4] = {0.f, 0.f, 0.f, 0.f};
-          each_tile([&] {
+          each_tile([&](int tile) {
+            if (TILE_SUMS) sums[0] = sums[1] = sums[2] = sums[3] = 0.f;
             load(gx, x);
             float u[K], ax[K];
             load(gu, u);
@@ -292,8 +316,9 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
             share(gr, r);
             share(gp[0], p);
             if (!ONE) store(grh, rh);
+            if (TILE_SUMS) grid.put(sums, tile);
           });
-          grid.sum(sums);
+          reduce4(sums);
           float rho = sums[1];
           const float stop2 = tol * tol * sums[0];
           conv = sums[1] <= stop2 || !(sums[0] > 1e-30f);
@@ -305,18 +330,20 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
             const float *vo = gv[m ? (m - 1) & 1 : 0], *po = gp[m ? (m - 1) & 1 : 0];
             float *vn = gv[m & 1], *pn = gp[m & 1];
             float sa[4] = {0.f, 0.f, 0.f, 0.f};
-            each_tile([&] {
+            each_tile([&](int tile) {
+              if (TILE_SUMS) sa[0] = sa[1] = sa[2] = sa[3] = 0.f;
               if (!ONE) {
-                load(grh, rh);
+                if (EARLY) load(grh, rh);
                 load(po, p);
                 if (m == 0) {
                   load(gr, r);
                 } else {
+                  load(gx, x);
+                  load(gq, q);
+                  if (!EARLY) advance_x(omega);
                   load(gs, r);
                   load(gt, t);
                   load(vo, v);
-                  load(gq, q);
-                  load(gx, x);
                 }
               }
               if (m == 0) {   // r and p are at hand
@@ -326,9 +353,9 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
                   const float rr = fmaf(-omega, __ldcg(gt + e), __ldcg(gs + e));
                   return fmaf(beta, fmaf(-omega, __ldcg(vo + e), __ldcg(po + e)), rr);
                 });
+                if (ONE || EARLY) advance(x, omega, q);
 #pragma unroll
                 for (int k = 0; k < K; ++k) {
-                  x[k] = fmaf(omega, q[k], x[k]);
                   r[k] = fmaf(-omega, t[k], r[k]);
                   p[k] = fmaf(beta, fmaf(-omega, v[k], p[k]), r[k]);
                 }
@@ -337,19 +364,24 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
               }
               put(P, p);
               precond_product(q, v);
+              if (!ONE && !EARLY) {
+                store(gq, q);
+                load(grh, rh);
+              }
 #pragma unroll
               for (int k = 0; k < K; ++k) {
                 sa[0] = fmaf(rh[k], v[k], sa[0]);
                 sa[1] = fmaf(r[k], r[k], sa[1]);
               }
               share(vn, v);
-              if (!ONE) {
+              if (!ONE && EARLY) {
                 store(gq, q);
                 if (m) store(gx, x);
               }
+              if (TILE_SUMS) grid.put(sa, tile);
             });
             open = false;
-            grid.sum(sa);
+            reduce4(sa);
             if (sa[1] <= stop2) {
               conv = true;
               break;
@@ -360,23 +392,26 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
             }
             alpha = rho / sa[0];
             float sb[4] = {0.f, 0.f, 0.f, 0.f};
-            each_tile([&] {
+            each_tile([&](int tile) {
+              if (TILE_SUMS) sb[0] = sb[1] = sb[2] = sb[3] = 0.f;
               if (!ONE) {
-                load(grh, rh);
+                if (EARLY) load(grh, rh);
+                load(gx, x);
+                load(gq, q);
+                if (!EARLY) advance_x(alpha);
                 load(gr, r);
                 load(vn, v);
-                load(gq, q);
-                load(gx, x);
               }
               halo(P, [&](size_t e) { return fmaf(-alpha, __ldcg(vn + e), __ldcg(gr + e)); });
-#pragma unroll
-              for (int k = 0; k < K; ++k) {
-                x[k] = fmaf(alpha, q[k], x[k]);
-                r[k] = fmaf(-alpha, v[k], r[k]);
-              }
+              if (ONE || EARLY) advance(x, alpha, q);
+              advance(r, -alpha, v);
               share(gs, r);
               put(P, r);
               precond_product(q, t);
+              if (!ONE && !EARLY) {
+                store(gq, q);
+                load(grh, rh);
+              }
 #pragma unroll
               for (int k = 0; k < K; ++k) {
                 sb[0] = fmaf(t[k], r[k], sb[0]);
@@ -385,12 +420,13 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
                 sb[3] = fmaf(rh[k], t[k], sb[3]);
               }
               share(gt, t);
-              if (!ONE) {
+              if (!ONE && EARLY) {
                 store(gq, q);
                 store(gx, x);
               }
+              if (TILE_SUMS) grid.put(sb, tile);
             });
-            grid.sum(sb);
+            reduce4(sb);
             open = true;
             omega = sb[1] > 0.f ? sb[0] / sb[1] : 0.f;
             const float rho_new = fmaf(-omega, sb[3], sb[2]);
@@ -402,15 +438,12 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
               rho = rho_new;
             }
           }
-          each_tile([&] {
+          each_tile([&](int) {
             if (!ONE) {
               load(gx, x);
               load(gq, q);
             }
-            if (open) {
-#pragma unroll
-              for (int k = 0; k < K; ++k) x[k] = fmaf(omega, q[k], x[k]);
-            }
+            if (open) advance(x, omega, q);
             store(gx, x);
           });
         }
@@ -419,10 +452,10 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
         iters_total += it;
         ++nsolves;
         nhist = nhist < 3 ? nhist + 1 : 3;
-        each_tile([&] { strip([&](int, size_t e) { gu[e] += gx[e]; }); });
+        each_tile([&](int) { strip([&](int, size_t e) { gu[e] += gx[e]; }); });
       }
       if (a.mode == SWEEP_PROP) {
-        each_tile([&] { strip([&](int, size_t e) { pit.out[e] = gu[e]; }); });
+        each_tile([&](int) { strip([&](int, size_t e) { pit.out[e] = gu[e]; }); });
         continue;
       }
       // correction u_{n+1} = F_n + (G_new - G_old_n), squares in FP32 (u_new - u_old of nearby
@@ -431,7 +464,7 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
       float* Un = a.U + (size_t)(n + 1) * MM;
       const float* Fn = a.Fb + (size_t)n * MM;
       float* Gn = a.Gold + (size_t)n * MM;
-      each_tile([&] {
+      each_tile([&](int) {
         strip([&](int, size_t e) {
           const float gnew = gu[e];
           if (a.mode == SWEEP_INIT) {
@@ -465,7 +498,7 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
         }
       };
       reduce(n0, n1);
-      double2* np = ca.npart + (size_t)group * 2 * kGridMaxBlocks + (n & 1) * kGridMaxBlocks;
+      double2* np = ca.npart + (n & 1) * ca.group_blocks;
       if (tid == 0) __stcg(np + grid.block, make_double2(n0, n1));
       grid.barrier();
       if (grid.block == 0) {   // (the slots alternate by slice: the next slice's barriers order their reuse)
@@ -501,7 +534,7 @@ __global__ void __launch_bounds__(kCgThreads, ONE ? 2 : 1) sweep_grid_kernel(con
 }
 
 // Blocks of the solver that the current device runs at once, measured once per device.
-template <bool ONE>
+template <bool ONE, int PER_SM>
 static int cg_blocks(int* out) {
   static std::mutex mu;
   static int known[64] = {};
@@ -511,7 +544,7 @@ static int cg_blocks(int* out) {
   int n = dev < 64 ? known[dev] : 0;
   if (!n) {
     int per_sm = 0, sms = 0;
-    BS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_grid_kernel<ONE>, kCgThreads, 0));
+    BS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_grid_kernel<ONE, PER_SM>, kCgThreads, 0));
     BS_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     n = std::min(per_sm * sms, kGridMaxBlocks);
     if (n < 1) return set_error(BS_ERR_CUDA, "coarse propagator: no block of the grid solver fits an SM");
@@ -521,37 +554,83 @@ static int cg_blocks(int* out) {
   return BS_OK;
 }
 
+// Layout of a launch of nst states.
+//  - Up to as many tiles as blocks are resident (about 770 nodes per axis): the layout with the least
+//    estimated time, rounds of states times microseconds per iteration.  A tile per block takes 12; with the
+//    tiles through the workspace it is 1 and 11.5 for every tile of a block, a quarter more where the
+//    groups' vectors exceed the L2 (fitted to 11.8 to 62 us at 512 to 700 nodes, one to eight groups).  A
+//    state that needs more than half of the resident blocks would leave the rest idle and the next
+//    states waiting: 7 states of 520 x 520, 2 steps, 12.0 ms in one group of 153 blocks and 6.9 in
+//    seven of 43; 64 of 512 x 512 56 and 49 ms.
+//  - Up to three tiles per SM, a block per SM: 22.8 us per iteration at 800 x 800, 25.1 with two.
+//  - Beyond, two blocks per SM (1024 x 1024: 25.4 us, 28.8 with one), in the groups with the least
+//    estimated time (8 states 65 and 49 ms).
+// The sums are added in the same order within each of the three ranges, so a state's result does not
+// depend on the others of its launch.
+enum CgKind { CG_ONE, CG_SHARED, CG_ALONE };   // a tile per block; several, two blocks or one block per SM
+struct CgLayout {
+  CgKind kind;
+  int group_blocks, groups;
+};
+static CgLayout cg_layout(int M, int tiles, int nst, const int (&blocks)[3]) {   // blocks: resident, by kind
+  constexpr int kMaxGroups = 8;
+  constexpr double kOneUs = 12.0, kPassUs = 1.0, kTileUs = 11.5, kL2Bytes = 110e6, kBeyondL2 = 1.25;
+  if (tiles > blocks[CG_ONE] && tiles <= 3 * blocks[CG_ALONE]) return {CG_ALONE, std::min(tiles, blocks[CG_ALONE]), 1};
+  auto rounds = [&](int groups) { return (double)((nst + groups - 1) / groups); };
+  CgLayout best = {};
+  double cost = 1e300;
+  if (tiles <= blocks[CG_ONE]) {
+    best = {CG_ONE, tiles, std::min(nst, blocks[CG_ONE] / tiles)};
+    cost = 0.97 * rounds(best.groups) * kOneUs;   // the others have to gain something
+  }
+  for (int g = 1; g <= std::min({nst, kMaxGroups, blocks[CG_SHARED]}); ++g) {
+    const int gb = std::min(tiles, blocks[CG_SHARED] / g);
+    double us = kPassUs + kTileUs * ((tiles + gb - 1) / gb);
+    if (g > 1 && 4.0 * kCgVectors * g * M * M > kL2Bytes) us *= kBeyondL2;
+    if (rounds(g) * us < cost) {
+      cost = rounds(g) * us;
+      best = {CG_SHARED, gb, g};
+    }
+  }
+  return best;
+}
+
 int launch_sweep_grid(const bs_grid* g, const ItemDesc& d, const SweepArgs& a, cudaStream_t s) {
   const int M = g->M;
   const size_t MM = (size_t)M * M;
   const int nst = a.mode == SWEEP_PROP && a.nprop > 0 ? a.nprop : 1;
   const int tiles = ((M + kCgW - 1) / kCgW) * ((M + kCgH - 1) / kCgH);
-  int blocks = 0;
-  int rc = cg_blocks<true>(&blocks);
-  if (rc) return rc;
-  const bool one = tiles <= blocks;
-  if (!one && (rc = cg_blocks<false>(&blocks))) return rc;
+  int blocks[3] = {}, rc;
+  if ((rc = cg_blocks<true, 2>(blocks + CG_ONE)) || (rc = cg_blocks<false, 2>(blocks + CG_SHARED)) ||
+      (rc = cg_blocks<false, 1>(blocks + CG_ALONE)))
+    return rc;
+  const CgLayout y = cg_layout(M, tiles, nst, blocks);
   CgArgs ca;
-  ca.group_blocks = std::min(tiles, blocks);
-  ca.groups = std::min(nst, blocks / ca.group_blocks);
-  // vectors, the groups' barrier words, norm partials
+  ca.tiles = tiles;
+  ca.group_blocks = y.group_blocks;
+  ca.groups = y.groups;
+  // vectors, the tiles' sums, norm partials, arrivals
   const size_t fbytes = ((size_t)ca.groups * kCgVectors * MM * sizeof(float) + 255) & ~(size_t)255;
-  const size_t pbytes = (size_t)ca.groups * sizeof(GridWords);
-  const size_t nbytes = (size_t)ca.groups * 2 * kGridMaxBlocks * sizeof(double2);
-  rc = ensure(const_cast<bs_grid*>(g)->ws_coarse, fbytes + pbytes + nbytes);
+  const size_t pbytes = (size_t)ca.groups * 2 * tiles * sizeof(float4);
+  const size_t nbytes = (size_t)2 * ca.group_blocks * sizeof(double2);
+  const size_t abytes = (size_t)ca.groups * kCgArrivalStride * sizeof(unsigned);
+  rc = ensure(const_cast<bs_grid*>(g)->ws_coarse, fbytes + pbytes + nbytes + abytes);
   if (rc) return rc;
   unsigned char* ws = static_cast<unsigned char*>(g->ws_coarse.ptr);
   ca.d = d;
   ca.a = a;
   ca.ws = reinterpret_cast<float*>(ws);
-  ca.words = reinterpret_cast<GridWords*>(ws + fbytes);
+  ca.partials = reinterpret_cast<float4*>(ws + fbytes);
   ca.npart = reinterpret_cast<double2*>(ws + fbytes + pbytes);
+  ca.arrivals = reinterpret_cast<unsigned*>(ws + fbytes + pbytes + nbytes);
   ca.M = M;
   ca.h = (float)(g->xmax / (M - 1));
-  BS_CUDA_TRY(cudaMemsetAsync(ca.words, 0, pbytes, s));
+  BS_CUDA_TRY(cudaMemsetAsync(ca.arrivals, 0, abytes, s));
   void* args[] = {&ca};
-  void* kern = one ? reinterpret_cast<void*>(sweep_grid_kernel<true>)
-                   : reinterpret_cast<void*>(sweep_grid_kernel<false>);
+  void* const kernels[] = {reinterpret_cast<void*>(sweep_grid_kernel<true, 2>),
+                           reinterpret_cast<void*>(sweep_grid_kernel<false, 2>),
+                           reinterpret_cast<void*>(sweep_grid_kernel<false, 1>)};
+  void* kern = kernels[y.kind];
   BS_CUDA_TRY(cudaLaunchCooperativeKernel(kern, dim3(ca.group_blocks * ca.groups),
                                           dim3(kCgThreads), args, 0, s));
   return BS_OK;

@@ -36,11 +36,16 @@ constexpr int kK3Tile = kK3HI * kK3HJ * kK3HK;
 constexpr int kK3Ring = kK3HI * kK3HJ - kK3Threads;                       // halo entries of an inner plane
 constexpr int kK3Halo = 2 * kK3HI * kK3HJ + kK3Planes * kK3Ring;          // halo entries of a tile
 
+struct K3Words {
+  float4 partials[2][kGridMaxBlocks];
+  unsigned arrivals;   // zero at launch
+};
+
 struct K3Args {
   F3Batch fb;          // item 0: in, out, hi, lo, tau0
   float *x, *r, *rh, *s, *t;
   float *p[2], *v[2];
-  GridWords* words;    // zero at launch
+  K3Words* words;
   int* status;         // bit 0: no convergence, bit 1: a barrier timed out; the launch returns at once if set
   int nsteps, maxit;
   float tol;
@@ -58,7 +63,7 @@ __global__ void __launch_bounds__(kK3Threads, 2) k3_solve_kernel(const __grid_co
   const int L0 = (kK3HJ + threadIdx.y + 1) * kK3HI + threadIdx.x + 1;   // tile index of the column's first plane
   constexpr int LZ = kK3HI * kK3HJ;
   const F3Coef& c = fb.c;
-  GridGroup<kK3Threads> grid{a.words, a.status, (int)blockIdx.x, (int)gridDim.x, tid};
+  GridGroup<kK3Threads> grid{&a.words->arrivals, a.words->partials[0], kGridMaxBlocks, a.status, (int)blockIdx.x, (int)gridDim.x, tid};
 
   int i0 = 0, j0 = 0, k0 = 0;
   // body(kk, e, pde) for every node of the thread's column in this block's tiles, after head()
@@ -335,7 +340,7 @@ static int k3_blocks(int* out) {
 constexpr int kK3Vectors = 11;
 size_t k3_workspace_bytes(int M) {
   const size_t n3 = (size_t)M * M * M;
-  return ((kK3Vectors * n3 * sizeof(float) + 255) & ~(size_t)255) + sizeof(GridWords) + 256;
+  return ((kK3Vectors * n3 * sizeof(float) + 255) & ~(size_t)255) + sizeof(K3Words) + 256;
 }
 int* k3_status(void* ws, int M) {
   return reinterpret_cast<int*>(static_cast<unsigned char*>(ws) + k3_workspace_bytes(M) - 256);
@@ -362,7 +367,7 @@ int coarse_propagate3_krylov(int M, double xmax, const bs_params3& p, const floa
   float** v[kK3Vectors] = {&it.hi, &it.lo, &a.x, &a.r, &a.rh, &a.s, &a.t, &a.p[0], &a.p[1], &a.v[0], &a.v[1]};
   for (int q = 0; q < kK3Vectors; ++q) *v[q] = f + q * n3;
   a.status = k3_status(ws, M);
-  a.words = reinterpret_cast<GridWords*>(reinterpret_cast<unsigned char*>(a.status) - sizeof(GridWords));
+  a.words = reinterpret_cast<K3Words*>(reinterpret_cast<unsigned char*>(a.status) - sizeof(K3Words));
   a.nsteps = nsteps;
   a.maxit = maxit;
   a.tol = (float)tol;
