@@ -189,9 +189,10 @@ int coarse_propagate(const bs_grid* g, int kind, const bs_pino* net, const bs_pa
 
 /* Coarse propagator G for B independent states at once (the same grid): as coarse_propagate
  * for item b with p[b], u_in[b] -> u_out[b], starting at tau0[b], over dtau_slice.
- *  kind = BS_COARSE_NUM: one thread-block cluster per state, one launch per run of
- *    consecutive items with equal parameters (at most 64 states each); on a grid with a
- *    coarse grid (bs_grid_set_coarse) the states are propagated one after another.
+ *  kind = BS_COARSE_NUM: one launch per run of consecutive items with equal parameters (at most
+ *    64 states each), a thread-block cluster per state up to M = 256, a group of blocks of one
+ *    cooperative launch beyond; on a grid with a coarse grid (bs_grid_set_coarse) the states are
+ *    propagated one after another.
  *  kind = BS_COARSE_PINO: the network on up to 128 states per launch chain (M <= 128: a cluster per
  *    state; else every product carries the states as extra rows or grid blocks); nsteps is ignored.
  * For concurrent solves or requests whose coarse steps are due together (a slice of each).

@@ -225,7 +225,7 @@ FineCounts grid_counts(bs_grid* g, const bs_params& p, double dtau) {
 }
 
 // Fine propagation of items whose Jacobi bound is too large for the sweep steppers: every
-// implicit step is solved by BiCGSTAB (the coarse solver), one cluster per state, in batched
+// implicit step is solved by BiCGSTAB (the coarse solver), a cluster or group of blocks per state, in batched
 // SWEEP_PROP launches of states that share their parameters and step size.
 int launch_krylov_fine(bs_grid* g, const ItemDesc* items, int n, int nsteps, cudaStream_t s) {
   auto same = [](const ItemDesc& a, const ItemDesc& b) {
@@ -441,7 +441,7 @@ int coarse_propagate_batched(const bs_grid* g, int kind, const bs_pino* net, con
     }
     return BS_OK;
   }
-  // one cluster per state, one launch per run of consecutive states with the same parameters
+  // one launch per run of consecutive states with the same parameters
   auto same = [](const bs_params& a, const bs_params& b) {
     return a.sigma1 == b.sigma1 && a.sigma2 == b.sigma2 && a.rho == b.rho && a.r == b.r && a.strike == b.strike &&
            a.w1 == b.w1 && a.w2 == b.w2 && a.payoff == b.payoff && a.strike2 == b.strike2 && a.cash == b.cash;

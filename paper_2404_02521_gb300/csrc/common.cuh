@@ -243,7 +243,7 @@ struct Options {
   int krylov_maxit = 400;
   int phase_timing = 0;
   int coarse_variant = -1;   // >= 0: force this coarse band variant; -1: measured per grid size
-  int fine_tile = 0;         // region layout of the fine tiles (M > 256): 0 auto, 1 or 2 forced
+  int fine_tile = 0;         // layout of the fine stepper (BS_OPT_FINE_TILE): 0 auto, 1 or 2 forced
 };
 extern Options g_opt;
 
@@ -273,8 +273,8 @@ struct bs_grid {
   double* dscal;               // device: scalar outputs (defect)
   double* dnorms;              // device: per-slice squared norms / defects
   bsp::Workspace ws_par;       // Parareal F / Gold buffers
-  bsp::Workspace ws_fine;      // tile fine stepper (M > 256): ping-pong hi, lo, increment
-  bsp::Workspace ws_coarse;    // global-memory coarse solver (M > 256): Krylov vectors
+  bsp::Workspace ws_fine;      // fine stepper over several regions (M > 256): ping-pong hi, lo, both increments
+  bsp::Workspace ws_coarse;    // coarse grid solver (M > 256): Krylov vectors, sums, barrier counters
   int coarse_variant = -1;     // band variant of the coarse sweep (-1: not chosen yet)
   int coarse_M = 0;            // numerical G on an Mc x Mc grid with resampling (0: this grid)
   bs_grid* coarse_grid = nullptr;   // that grid (created on first use)
@@ -297,7 +297,7 @@ int launch_payoff(const bs_grid* g, const ItemDesc& d, float* u, cudaStream_t s)
 FineCounts grid_counts(bs_grid* g, const bs_params& p, double dtau);
 // Coarse numerical propagation / Parareal serial sweep (see coarse.cu).
 enum { SWEEP_PROP = 0, SWEEP_INIT = 1, SWEEP_ITER = 2 };
-// Independent states propagated by one batched SWEEP_PROP launch (one cluster each): the
+// Independent states propagated by one batched SWEEP_PROP launch (a cluster or group each): the
 // Krylov fine propagator for steps whose Jacobi bound is too large.
 constexpr int kMaxProp = 64;
 struct PropItem {
@@ -321,7 +321,7 @@ struct SweepArgs {
   int* status;
   double tol;           // relative residual of the Krylov solve
   int maxit;
-  int nprop;            // SWEEP_PROP: > 0 -> cluster blockIdx.y propagates prop[blockIdx.y]
+  int nprop;            // SWEEP_PROP: > 0 -> a cluster (M <= 256: blockIdx.y) or group per prop[]
   PropItem prop[kMaxProp];
   // INIT / ITER in chunks: with n_end > 0 the launch runs slices n_begin .. n_end-1 only,
   // starting from U[n_begin] (written by the chunk before) unless n_begin == n_first; the

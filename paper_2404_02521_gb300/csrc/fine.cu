@@ -6,10 +6,11 @@
 //   (I - dtau R_h) d = dtau R_h w,   w = u^m inside, g(tau^{m+1}) on the far edges,
 // with d = 0 on the far edges.  It is solved by Jacobi sweeps
 //   d <- (b + sum_k c_k d_k) / (1 + sum_k c_k + r dtau),   b = dtau R_h w,
-// started from the previous step's increment.  The Gershgorin bound q < 1 of the system
+// started from zero in the first step of a call, from the previous increment in the second and from
+// the extrapolation of the previous two after that.  The Gershgorin bound q < 1 of the system
 // (checked on the host) makes every sweep a max-norm contraction by q; the sweep count is
-// chosen so that q^sweeps is below a target (2^-22 for the first, cold-started step of a
-// launch, 2^-10 for the warm-started steps after it).  The state is a compensated
+// chosen so that q^sweeps is below a target (2^-22, 2^-10, 2^-6 up to step 15 and 1/2 from there)
+// and extrapolated starts converge (capi.cu: extrap_stable).  The state is a compensated
 // pair (hi, lo): u = hi + lo, updated by an error-free two-sum, so that increments below half
 // an ulp of u are not lost over tens of thousands of steps; b is evaluated from hi.
 #include <algorithm>

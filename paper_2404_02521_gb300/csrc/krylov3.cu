@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(kK3Threads, 2) k3_solve_kernel(const __grid_co
   GridGroup<kK3Threads> grid{&a.words->arrivals, a.words->partials[0], kGridMaxBlocks, a.status, (int)blockIdx.x, (int)gridDim.x, tid};
 
   int i0 = 0, j0 = 0, k0 = 0;
-  // body(kk, e, pde) for every node of the thread's column in this block's tiles, after head()
+  // body() for each of this block's tiles, whose first node is (i0, j0, k0)
   auto each_tile = [&](auto&& body) {
     for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
       const int tk = tile / (tiles_i * tiles_j), rem = tile - tk * (tiles_i * tiles_j), tj = rem / tiles_i;

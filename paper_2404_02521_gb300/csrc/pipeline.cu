@@ -3,8 +3,8 @@
 // Eq. (parareal) needs F(u_n^k) only when the sweep of iteration k-1 has produced u_n^k, so F
 // and the serial coarse sweep need not alternate as whole phases.  Each sweep is split into
 // chunks of S consecutive slices, launched one after another on an internal stream of the
-// highest priority (so that a sweep chunk's 16-CTA cluster is placed before an F chunk that
-// becomes ready at the same moment); the F launch of a chunk goes to a low-priority stream
+// highest priority (so that a sweep chunk's 16-CTA cluster, up to 256 x 256, is placed before an F
+// chunk that becomes ready at the same moment); the F launch of a chunk goes to a low-priority stream
 // and waits (cudaStreamWaitEvent) for the sweep chunk that finished its input states.  Both
 // streams start after the caller's stream and the caller's stream waits for both at the end.
 // The sweep chunk of iteration k waits for the F chunk of iteration k over the same slices.
@@ -13,7 +13,10 @@
 // copies its last state into a snapshot (two sets, by iteration parity) that F chunk c reads.
 // F of iteration k+1 is launched before the host has read the defect of iteration k
 // (speculatively: it writes only the F workspace, and is wasted if iteration k converged), so
-// it runs on the SMs the 16-CTA coarse cluster leaves free while the sweep continues.  All ordering is between whole kernels through stream
+// it runs on the SMs the 16-CTA coarse cluster leaves free while the sweep continues.  Beyond 256 x 256
+// the sweep is a cooperative launch over most SMs, for which an F launch of 8-column tiles, whose
+// CTAs hold an SM's registers, leaves no room: the two take turns, launch by launch (512 x 512, N = 16
+// with G on that grid: 447 ms; 896 with the sweep on one cluster beside F).  All ordering is between whole kernels through stream
 // events; no kernel waits on another.  Results: the same Parareal iteration; on the state grid
 // the coarse solves restart their extrapolated initial guesses at chunk boundaries, so G agrees
 // with the unchunked sweep to the Krylov tolerance, not bitwise; with G on a coarse grid every
@@ -38,8 +41,9 @@ struct PipeState {
 static int pipe_state(bs_grid* g, int chunks, PipeState** out) {
   if (!g->pipe) {
     PipeState* ps = new PipeState();
-    // A sweep chunk's cluster needs 16 SMs of one GPC; when it and an F chunk become ready
-    // together, the higher stream priority places the cluster first.
+    // A sweep chunk's cluster needs 16 SMs of one GPC (its cooperative launch beyond 256 x 256 all of
+    // its blocks at once); when it and an F chunk become ready together, the higher stream priority
+    // places it first.
     int lo = 0, hi = 0;
     cudaDeviceGetStreamPriorityRange(&lo, &hi);
     if (cudaStreamCreateWithPriority(&ps->ss, cudaStreamNonBlocking, hi) != cudaSuccess ||
@@ -96,7 +100,8 @@ bool pipeline_eligible(int N) { return N >= 8; }
 // second wave, or an F wave that leaves no GPC for the sweep's cluster, stalls the sweep --
 // on the 256 x 256 workload chunks of 16 slices took 60 ms per solve, of 12 slices 48, and the
 // 13 of this rule 44.
-// At most a quarter of the slices, so that F starts early and the sweep drains soon.
+// At most a quarter of the slices, so that F starts early and the sweep drains soon (beyond 256 x 256
+// that alone).
 int pipeline_chunk(bs_grid* g, const ItemDesc& dc, int N, cudaStream_t s, int* S) {
   int quarter = (N + 3) / 4;
   const int cap = fine_cluster_capacity(g);
